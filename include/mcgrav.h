@@ -165,24 +165,21 @@ typedef struct {
                                 walk options: capture each batch of rounds (walk,
                                 reductions, result copies) and launch it as one graph
                                 (default 1) */
-    int32_t migrate;         /* mixed walk: once the work list is used up, warps with
-                                few walks left hand them to warps with free lanes
-                                through a pool in work_dev (default 1).  Results do
-                                not depend on it for piecewise-constant densities;
-                                for a voxel grid the single-precision partial sums
-                                are flushed at other steps (rounding only).       */
+    int32_t migrate;         /* mixed walk: 1 (default) lets fault_unpublished act;
+                                no effect otherwise: once the work list is used up a
+                                warp runs its last walks with several lanes each
+                                instead of handing them to other warps             */
     int32_t fault_unpublished;/* failure-detection test hook, 0..255 (default 0):
-                                the launch starts with this many migration-pool
-                                slots reserved but never published, as if a warp
-                                had died between its reservation and its store.
-                                A warp that claims one waits a bounded time
-                                (about 0.1-1 s) for it, gives up, and the walk
-                                reports MCG_ERR_TIMEOUT; every real walk still
-                                finishes.  Needs the mixed walk with migrate = 1. */
-    int32_t spill_max;       /* mixed walk with migrate = 1: once the work list is used
-                                up, a warp with at most this many live walks (1..32,
-                                default 24; 0 = default) hands them to warps with free
-                                lanes (mcg_autotune picks it)                     */
+                                the launch starts with this many slots of a
+                                hand-over pool reserved but never published, as if
+                                a warp had died between its reservation and its
+                                store.  A warp without walks that claims one waits a
+                                bounded time (about 0.1-1 s) for it, gives up, and
+                                the walk reports MCG_ERR_TIMEOUT; every real walk
+                                still finishes.  Needs the mixed walk with
+                                migrate = 1.                                       */
+    int32_t spill_max;       /* accepted (0..32, default 24; 0 = default) and without
+                                effect, see migrate                                */
 } mcg_options;
 
 /* Per-station outputs (caller-owned, length S; any pointer may be NULL). */
@@ -248,8 +245,7 @@ MCG_API int mcgrav_solve(const mcg_domain* domain, const mcg_density* density, c
  *   work_dev    : DEVICE scratch of mcg_walk_work_bytes(S, N, precision)
  *                 bytes (the mixed walk stores each copy's exit record
  *                 there and a second kernel evaluates the exits; it also
- *                 holds the migration pool and its counters, reset by this
- *                 call); may be NULL when that size is 0.  Caller-owned,
+ *                 holds fault_unpublished's slots); may be NULL when that size is 0.  Caller-owned,
  *                 256-byte aligned.
  *   status_dev  : DEVICE int32, OR-ed with (1 << status) for every path that
  *                 hit the step cap, started outside Omega or produced a
@@ -296,8 +292,7 @@ MCG_API size_t mcg_walk_work_bytes(int64_t S, int64_t N, int32_t precision);
  *     serialise them.
  *   - The array's address is cached per device after the first call; a
  *     device reset (cudaDeviceReset) after that call is not supported.
- *   - opts->migrate is ignored: the array holds no migration pool, so each
- *     warp keeps its walks to the end (same results, longer exit-time tail).
+ *   - opts->fault_unpublished is ignored.
  * Asynchronous on opts->stream like mcg_walk. */
 MCG_API int mcg_walk_static(const mcg_domain* domain, const mcg_density* density, const mcg_boundary* boundary,
                             const double* stations_dev, int64_t S, int64_t p0, int64_t N, double dt, uint64_t seed,
@@ -338,13 +333,10 @@ MCG_API int mcg_states_merge(const mcg_station_state* parts, int64_t R, int64_t 
  *   1. opts->block (64, 96, 128) on short walks of the given stations capped
  *      at 2048 RNG-steps (the stepping rate, every lane busy; all walks of a
  *      warp end together, so the refill policy plays no part);
- *   2. mixed walk: opts->refill_min (1, 4, 16) x opts->spill_max (8, 16, 24,
- *      32; with migrate = 1 only) on uncapped walks, two per resident lane,
- *      whose launch ends in the exit-time tail: lanes free up at random steps
- *      and walk migration shortens the tail.  The defaults (refill 1, the
- *      incoming spill threshold, 24 when unset) stay unless another pair is
- *      more than 1 % faster (skipped for the FP64 walk; stops early, keeping
- *      them, once one launch takes over 2 s).
+ *   2. mixed walk: opts->refill_min (1, 4, 16) on uncapped walks, two per
+ *      resident lane, where lanes free up at random steps.  The default (1)
+ *      stays unless another is more than 1 % faster (skipped for the FP64
+ *      walk; stops early, keeping it, once one launch takes over 2 s).
  * stations_dev: DEVICE, S x 3.  Blocking; allocates and frees a scratch
  * area of mcg_walk's size for the larger of the two stages. */
 MCG_API int mcg_autotune(const mcg_domain* domain, const mcg_density* density, const mcg_boundary* boundary,

@@ -110,16 +110,14 @@ void bind_work(WalkParams& P, void* work, bool migrate)
     const WorkLayout L = work_layout((size_t)P.total);
     unsigned char* w = (unsigned char*)work;
     P.frec = (float*)(w + L.frec);
-    if (migrate && L.cap > 0) {
+    if (migrate && P.fault_unpublished && L.cap > 0) {
         P.pool = w + L.pool;
         P.pool_ready = (uint32_t*)(w + L.ready);
         P.pool_ctr = (unsigned long long*)(w + L.ctr);
-        P.pool_cap = L.cap;
     } else {
         P.pool = nullptr;
         P.pool_ready = nullptr;
         P.pool_ctr = nullptr;
-        P.pool_cap = 0;
     }
 }
 
@@ -286,7 +284,6 @@ int make_params(const mcg_domain* D, const mcg_density* R, const mcg_boundary* B
     if (o->refill_min < 0 || o->refill_min > 32) return set_error(MCG_ERR_ARG, "refill_min must be in [0, 32]");
     P.refill_min = o->refill_min > 0 ? o->refill_min : 1;
     if (o->spill_max < 0 || o->spill_max > 32) return set_error(MCG_ERR_ARG, "spill_max must be in [0, 32]");
-    P.spill_max = o->spill_max > 0 ? o->spill_max : 24;
     P.bridge_k = -2.0 / (P.sd * P.sd);
     P.bridge_k_f = (float)P.bridge_k;
     // Conservative boxes for the walk's common step (all copies inside, no

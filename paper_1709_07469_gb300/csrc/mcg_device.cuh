@@ -213,6 +213,29 @@ __device__ __forceinline__ void voxel_cell(const WalkParams& P, float x, float y
     fr = __fsub_rn(tz, __fsub_rn(vz, kFloorMagic));
 }
 
+// Copies (x, y, z), (x, y, z + h), (x, y, z - h) in the support of a density
+// that is rho0 or 0: bit c for copy c (the tests of rho3_f32 below).
+template <int RHO>
+__device__ __forceinline__ unsigned support3_f32(const WalkParams& P, float x, float y, float z, float h)
+{
+    unsigned in;
+    if constexpr (RHO == MCG_RHO_SPHERE) {
+        const float dx = __fsub_rn(x, P.sc_f[0]), dy = __fsub_rn(y, P.sc_f[1]), dz = __fsub_rn(z, P.sc_f[2]);
+        const float q = __fmaf_rn(dx, dx, __fmul_rn(dy, dy));
+        const float zb = __fadd_rn(dz, h), zc = __fsub_rn(dz, h);
+        in = (__fmaf_rn(dz, dz, q) < P.srad2_f) ? 1u : 0u;
+        in |= (__fmaf_rn(zb, zb, q) < P.srad2_f) ? 2u : 0u;
+        in |= (__fmaf_rn(zc, zc, q) < P.srad2_f) ? 4u : 0u;
+    } else {
+        const bool inxy = x >= P.plo_f[0] && x < P.phi_f[0] && y >= P.plo_f[1] && y < P.phi_f[1];
+        const float zb = __fadd_rn(z, h), zc = __fsub_rn(z, h);
+        in = (inxy && z >= P.plo_f[2] && z < P.phi_f[2]) ? 1u : 0u;
+        in |= (inxy && zb >= P.plo_f[2] && zb < P.phi_f[2]) ? 2u : 0u;
+        in |= (inxy && zc >= P.plo_f[2] && zc < P.phi_f[2]) ? 4u : 0u;
+    }
+    return in;
+}
+
 // Density at the three common-random-number copies (x, y, z), (x, y, z+h),
 // (x, y, z-h): the x / y part is computed once.  Every rounding step is
 // explicit (no contraction left to the compiler), so the walk kernel and the
@@ -222,19 +245,11 @@ template <int RHO>
 __device__ __forceinline__ void rho3_f32(const WalkParams& P, const ModelRef& M, float x, float y, float z, float h,
                                          float& ra, float& rb, float& rc)
 {
-    if constexpr (RHO == MCG_RHO_SPHERE) {
-        const float dx = __fsub_rn(x, P.sc_f[0]), dy = __fsub_rn(y, P.sc_f[1]), dz = __fsub_rn(z, P.sc_f[2]);
-        const float q = __fmaf_rn(dx, dx, __fmul_rn(dy, dy));
-        const float za = dz, zb = __fadd_rn(dz, h), zc = __fsub_rn(dz, h);
-        ra = (__fmaf_rn(za, za, q) < P.srad2_f) ? P.rho0_f : 0.0f;
-        rb = (__fmaf_rn(zb, zb, q) < P.srad2_f) ? P.rho0_f : 0.0f;
-        rc = (__fmaf_rn(zc, zc, q) < P.srad2_f) ? P.rho0_f : 0.0f;
-    } else if constexpr (RHO == MCG_RHO_PRISM) {
-        const bool inxy = x >= P.plo_f[0] && x < P.phi_f[0] && y >= P.plo_f[1] && y < P.phi_f[1];
-        const float zb = __fadd_rn(z, h), zc = __fsub_rn(z, h);
-        ra = (inxy && z >= P.plo_f[2] && z < P.phi_f[2]) ? P.rho0_f : 0.0f;
-        rb = (inxy && zb >= P.plo_f[2] && zb < P.phi_f[2]) ? P.rho0_f : 0.0f;
-        rc = (inxy && zc >= P.plo_f[2] && zc < P.phi_f[2]) ? P.rho0_f : 0.0f;
+    if constexpr (RHO == MCG_RHO_SPHERE || RHO == MCG_RHO_PRISM) {
+        const unsigned in = support3_f32<RHO>(P, x, y, z, h);
+        ra = (in & 1u) ? P.rho0_f : 0.0f;
+        rb = (in & 2u) ? P.rho0_f : 0.0f;
+        rc = (in & 4u) ? P.rho0_f : 0.0f;
     } else if constexpr (RHO == MCG_RHO_VOXEL) {
         int ix, iy, iz;
         float fr;

@@ -46,7 +46,7 @@ struct WalkParams {
     double dt, sd, h, two_pi_G;
     float sd_f, h_f, lnscale_f;    // lnscale_f = -2 ln 2 sd^2
     int32_t crn, clip, bridge, refill_min;
-    int32_t spill_max;             // a warp with at most this many live walks hands them over
+    int32_t quota;                 // walks a warp holds at most (launch_walk)
     float bridge_k_f;              // -2 / (sigma^2 dt), single precision
     double bridge_k;               // -2 / (sigma^2 dt)
     int64_t max_steps;
@@ -62,14 +62,11 @@ struct WalkParams {
     unsigned long long* counter;
     float* frec;                   // mixed walk: exit records (32 bytes per copy per item), or null
     volatile int32_t* cancel;
-    // mixed walk, migration of walks between warps once the work list is used
-    // up (null pool: off).  pool: kPoolEntryBytes per slot; pool_ready: one
-    // flag per slot; pool_ctr: [0] slots reserved, [1] slots claimed, [2]
-    // warps gone.
+    // mixed walk, failure-detection hook (null pool: off).  pool_ready: one
+    // flag per hand-over slot; pool_ctr: [0] slots reserved, [1] slots claimed.
     unsigned char* pool;
     uint32_t* pool_ready;
     unsigned long long* pool_ctr;
-    unsigned long long pool_cap;
     uint32_t fault_unpublished;    // host side: pool slots reserved and never published
     // multi-request launch: segment table (device) sorted by begin, or null
     const struct WalkSeg* seg;
@@ -109,21 +106,23 @@ constexpr size_t kPoolEntryBytes = 80;
 constexpr unsigned long long kPoolMaxSlots = 1ull << 19;
 
 // Offsets inside the mixed walk's scratch of n = S * N items (mcg_api.cu):
-// exit records, migration pool, ready flags, pool counters.
+// exit records, hand-over slots (not used), ready flags, counters (the
+// failure-detection hook's).
 constexpr size_t kExitRecordBytes = 32;
 struct WorkLayout {
     size_t frec, pool, ready, ctr, total;
     unsigned long long cap;
 };
 WorkLayout work_layout(size_t n);
-// Points P's mixed-walk buffers into `work` (layout above); migration on/off.
+// Points P's mixed-walk buffers into `work` (layout above); `migrate`: with the
+// failure-detection hook, where the options ask for it.
 void bind_work(WalkParams& P, void* work, bool migrate);
 // mcgrav_solve's workspace parts (mcg_api.cu).
 size_t solve_shared_bytes(int64_t S);
 size_t solve_set_bytes(int64_t S, int64_t batch);
 // Zeroes the work counter, marks every item "no result" (exit records of the
-// mixed walk, per-path values of the FP64 walk, steps 0) and, with migration,
-// zeroes the pool's flags and counters.
+// mixed walk, per-path values of the FP64 walk, steps 0) and, with the
+// failure-detection hook, sets up its flags and counters.
 cudaError_t reset_walk(const WalkParams& P, cudaStream_t st);
 
 // Kernel launchers (mcg_walk.cu).

@@ -26,9 +26,8 @@ int mcg_autotune(const mcg_domain* domain, const mcg_density* density, const mcg
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     // Stage 1 (stepping rate): about 2.6e5 capped walks (a few per lane of the
-    // persistent grid), at most 2048 per station.  Stage 2 (exit-time tail):
-    // uncapped walks, two per resident lane, so the launch ends in the tail
-    // that migration shortens.
+    // persistent grid), at most 2048 per station.  Stage 2: uncapped walks,
+    // two per resident lane.
     int64_t N1 = (262144 + S - 1) / S;
     if (N1 > 2048) N1 = 2048;
     const int kind = (P.rho_kind == MCG_RHO_VOXEL && P.zq) ? kRhoVoxelPacked : P.rho_kind;
@@ -77,7 +76,7 @@ int mcg_autotune(const mcg_domain* domain, const mcg_density* density, const mcg
     // cap together, so the refill policy plays no part here); one warm-up
     // launch, then the median of three launches per candidate.
     const int blocks[3] = {64, 96, 128};
-    int best_block = 128, best_refill = 1, best_spill = P.spill_max;
+    int best_block = 128, best_refill = 1;
     rc = MCG_OK;
     P.N = N1;
     P.total = (unsigned long long)S * (unsigned long long)N1;
@@ -97,51 +96,35 @@ int mcg_autotune(const mcg_domain* domain, const mcg_density* density, const mcg
                 best_block = blocks[bi];
             }
     }
-    // Stage 2 (mixed walk): refill threshold x spill threshold, on uncapped
-    // walks whose launch ends in the exit-time tail (refills happen as walks
-    // exit at random steps, and migration shortens the tail).  One timing per
-    // candidate is noisy there: the median of three decides, and the default
-    // (refill 1, the options' spill threshold) stays unless another pair is
-    // faster by more than 1 %.
+    // Stage 2 (mixed walk): refill threshold, on uncapped walks (refills
+    // happen as walks exit at random steps).  One timing per candidate is
+    // noisy there: the median of three decides, and the default (refill 1)
+    // stays unless another is faster by more than 1 %.
     if (rc == MCG_OK && o.precision == MCG_MIXED) {
         P.max_steps = opts->max_steps;
         P.N = N2;
         P.total = (unsigned long long)S * (unsigned long long)N2;
         bind_work(P, w, o.migrate != 0);
         const int refills[3] = {1, 4, 16};
-        const int spills_m[4] = {8, 16, 24, 32};
-        const int dflt_spill = P.spill_max;
-        const int* spills = o.migrate ? spills_m : &dflt_spill;
-        const int ns = o.migrate ? 4 : 1;
-        float t2[3][4][3];
+        float t2[3][3];
         P.refill_min = 1;
         const float warm = timed(best_block);
         if (warm < 0.0f) rc = set_error(MCG_ERR_CUDA, "autotune launch: %s", cudaGetErrorString(e));
-        const bool too_long = warm > 2000.0f;  // very long walks: keep the defaults
+        const bool too_long = warm > 2000.0f;  // very long walks: keep the default
         for (int rep = 0; rep < 3 && rc == MCG_OK && !too_long; ++rep)
-            for (int ri = 0; ri < 3 && rc == MCG_OK; ++ri)
-                for (int si = 0; si < ns && rc == MCG_OK; ++si) {
-                    P.refill_min = refills[ri];
-                    P.spill_max = spills[si];
-                    t2[ri][si][rep] = timed(best_block);
-                    if (t2[ri][si][rep] < 0.0f)
-                        rc = set_error(MCG_ERR_CUDA, "autotune launch: %s", cudaGetErrorString(e));
-                }
-        best_spill = dflt_spill;
+            for (int ri = 0; ri < 3 && rc == MCG_OK; ++ri) {
+                P.refill_min = refills[ri];
+                t2[ri][rep] = timed(best_block);
+                if (t2[ri][rep] < 0.0f) rc = set_error(MCG_ERR_CUDA, "autotune launch: %s", cudaGetErrorString(e));
+            }
         if (rc == MCG_OK && !too_long) {
-            float med_dflt = -1.0f;
-            for (int si = 0; si < ns; ++si)
-                if (spills[si] == dflt_spill) med_dflt = med3(t2[0][si]);
-            float best2 = med_dflt > 0.0f ? med_dflt / 1.01f : 1e30f;
-            for (int ri = 0; ri < 3; ++ri)
-                for (int si = 0; si < ns; ++si)
-                    if (med3(t2[ri][si]) < best2) {
-                        best2 = med3(t2[ri][si]);
-                        best_refill = refills[ri];
-                        best_spill = spills[si];
-                    }
+            float best2 = med3(t2[0]) / 1.01f;
+            for (int ri = 1; ri < 3; ++ri)
+                if (med3(t2[ri]) < best2) {
+                    best2 = med3(t2[ri]);
+                    best_refill = refills[ri];
+                }
         }
-        if (too_long) best_spill = opts->spill_max > 0 ? opts->spill_max : 24;
     }
     cudaEventDestroy(a);
     cudaEventDestroy(b);
@@ -149,7 +132,7 @@ int mcg_autotune(const mcg_domain* domain, const mcg_density* density, const mcg
     if (rc) return rc;
     opts->block = best_block;
     opts->refill_min = best_refill;
-    opts->spill_max = best_spill;
+    if (opts->spill_max <= 0) opts->spill_max = 24;
     return MCG_OK;
 }
 

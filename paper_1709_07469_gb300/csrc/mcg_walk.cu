@@ -14,10 +14,11 @@
 //    rounding of the transcendental functions.
 //  * walk_mixed_kernel: single-precision stepping, random-number transform
 //    and density lookup; the source integral keeps single-precision partial
-//    sums over at most 64 steps which are flushed into a double accumulator;
+//    sums over at most 64 steps which are flushed into a double accumulator
+//    (an exact count where the density is rho0 or 0);
 //    the exit-segment clip, the boundary value and the per-path estimate are
-//    double precision and run in exit_mixed_kernel.  Once the work list is
-//    used up, walks migrate from sparse warps to warps with free lanes.
+//    double precision and run in exit_mixed_kernel.  Where a warp has few
+//    walks (small launches, the exit-time tail) its lanes share them.
 //
 // Launch shape: 128 threads, at least MCG_MIXED_MINB blocks per SM (the
 // register bound that gave the best rate; the grid is sized from the
@@ -41,26 +42,26 @@ constexpr unsigned kFull = 0xffffffffu;
 constexpr double kNaN = __builtin_nan("");
 
 
-// Claims new items for the lanes of this warp that are free.  Returns the
-// claimed item in `item`; lanes beyond the end of the work list become
-// `exhausted`.
-__device__ __forceinline__ bool refill(const WalkParams& P, bool busy, bool& exhausted,
+// Claims new items for free lanes of this warp while it holds fewer than
+// `quota` walks.  Returns true on the lanes that got one (in `item`); sets
+// the warp-uniform `drained` once the work list has no more.
+__device__ __forceinline__ bool refill(const WalkParams& P, bool busy, unsigned quota, bool& drained,
                                        unsigned long long& item)
 {
-    const unsigned want = __ballot_sync(kFull, !busy && !exhausted);
-    if (want == 0u) return false;
+    const unsigned freem = __ballot_sync(kFull, !busy);
+    const unsigned live = 32u - (unsigned)__popc(freem);
+    if (drained || live >= quota) return false;
     const int lane = threadIdx.x & 31;
-    const int leader = __ffs(want) - 1;
+    const unsigned rank = (unsigned)__popc(freem & ((1u << lane) - 1u));
+    const bool want = !busy && rank < quota - live;
+    const unsigned wantm = __ballot_sync(kFull, want);
+    const int leader = __ffs(wantm) - 1;
     unsigned long long base = 0ull;
-    if (lane == leader) base = atomicAdd(P.counter, (unsigned long long)__popc(want));
+    if (lane == leader) base = atomicAdd(P.counter, (unsigned long long)__popc(wantm));
     base = __shfl_sync(kFull, base, leader);
-    if (busy || exhausted) return false;
-    item = base + (unsigned long long)__popc(want & ((1u << lane) - 1u));
-    if (item >= P.total) {
-        exhausted = true;
-        return false;
-    }
-    return true;
+    drained = base + (unsigned long long)__popc(wantm) >= P.total;
+    item = base + rank;  // the wanting lanes are the first of the free ones
+    return want && item < P.total;
 }
 
 // A station whose walk copies are not all strictly inside Omega gets NaN
@@ -101,27 +102,16 @@ __device__ __forceinline__ bool cancelled(const WalkParams& P)
 }
 
 // ---------------------------------------------------------------------------
-// Migration of walks between warps (mixed walk).  Once the work list is used
-// up, a warp's lanes empty one by one as its walks exit, and a warp with a
-// few long walks left would keep issuing instructions for 32 lanes to the
-// end.  Such a warp (at most P.spill_max walks live, migration on) writes its
-// walks to the pool and leaves; warps with free lanes claim pooled walks.
-// A walk's state is all of it: the random streams are keyed by (station,
-// path, step), so where a walk continues does not change its numbers.
-//   reserve: CAS on pool_ctr[0] below pool_cap; entries written, then the
-//            slot's ready flag set with release semantics;
-//   claim  : CAS on pool_ctr[1] below pool_ctr[0]; acquire on the ready flag
-//            (a bounded wait: the producer is a running warp between its
-//            reservation and its store, so the flag comes);
-//   leave  : a warp with no walks adds 1 to pool_ctr[2]; the last warp to
-//            leave (count = all warps of the grid) sees every earlier spill
-//            and, if the pool still holds walks, takes them over.
-// Each warp spills at most once, so slots are never reused.
+// Bounded wait on a hand-over slot (failure-detection hook).  Walks stay in
+// the warp that claimed them: once the work list is used up a warp runs the
+// walks it has left as strips (below), which is faster than handing them to
+// other warps (prism ore body, 30 x 8192 paths: 162 ms against 190 ms; voxel
+// survey, 256 x 512: 5.8 against 11.6 ms).  mcg_options.fault_unpublished
+// starts a launch with slots of the hand-over pool reserved and never
+// published, as by a warp that died between the two; a warp without walks
+// claims one, waits a bounded time for its ready flag and reports
+// MCG_ERR_TIMEOUT.  pool_ctr[0]: slots reserved, [1]: slots claimed.
 // ---------------------------------------------------------------------------
-#ifndef MCG_SPILL_BACKLOG
-#define MCG_SPILL_BACKLOG 64
-#endif
-constexpr unsigned long long kSpillBacklog = MCG_SPILL_BACKLOG;  // ... while fewer pooled walks wait
 constexpr int kReadySpin = 1 << 20;                   // bounded wait for a ready flag (~0.1 s)
 
 __device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long long* a)
@@ -136,57 +126,18 @@ __device__ __forceinline__ uint32_t ld_acquire_u32(const uint32_t* a)
     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(a) : "memory");
     return v;
 }
-__device__ __forceinline__ void st_release_u32(uint32_t* a, uint32_t v)
-{
-    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(a), "r"(v) : "memory");
-}
 
-// Leader: claims up to `want` pooled walks; returns the count, first slot in base.
-__device__ __forceinline__ unsigned pool_take(const WalkParams& P, unsigned want, unsigned long long& base)
+// One thread: claims a reserved slot, if there is one, and waits for it.
+__device__ __forceinline__ void pool_wait(const WalkParams& P)
 {
-    for (int t = 0; t < 32; ++t) {
-        const unsigned long long r = ld_acquire_u64(P.pool_ctr);
-        const unsigned long long c = ld_acquire_u64(P.pool_ctr + 1);
-        if (c >= r) return 0u;
-        const unsigned long long k = (r - c) < want ? (r - c) : want;
-        if (atomicCAS(P.pool_ctr + 1, c, c + k) == c) {
-            base = c;
-            return (unsigned)k;
-        }
+    const unsigned long long c = ld_acquire_u64(P.pool_ctr + 1);
+    if (c >= ld_acquire_u64(P.pool_ctr) || atomicCAS(P.pool_ctr + 1, c, c + 1ull) != c) return;
+    uint32_t ready = 0u;
+    for (int i = 0; i < kReadySpin && !ready; ++i) {
+        ready = ld_acquire_u32(P.pool_ready + c);
+        if (!ready) __nanosleep(64);
     }
-    return 0u;
-}
-
-// Leader: reserves n slots if the pool has room and few walks wait there.
-__device__ __forceinline__ bool pool_reserve(const WalkParams& P, unsigned n, unsigned long long& base)
-{
-    for (int t = 0; t < 32; ++t) {
-        const unsigned long long r = ld_acquire_u64(P.pool_ctr);
-        const unsigned long long c = ld_acquire_u64(P.pool_ctr + 1);
-        if (r - c >= kSpillBacklog || r + n > P.pool_cap) return false;
-        if (atomicCAS(P.pool_ctr, r, r + n) == r) {
-            base = r;
-            return true;
-        }
-    }
-    return false;
-}
-
-// Leader: records that this warp has no walks.  Returns false when it was
-// the last warp of the grid to leave and walks are still pooled: it must
-// take them over.
-__device__ __forceinline__ bool pool_leave(const WalkParams& P, bool stop)
-{
-    __threadfence();
-    const unsigned long long warps = (unsigned long long)gridDim.x * (blockDim.x >> 5);
-    const unsigned long long prev = atomicAdd(P.pool_ctr + 2, 1ull);
-    if (stop || prev + 1ull != warps) return true;
-    __threadfence();
-    if (ld_acquire_u64(P.pool_ctr + 1) < ld_acquire_u64(P.pool_ctr)) {
-        atomicAdd(P.pool_ctr + 2, ~0ull);  // -1: still here
-        return false;
-    }
-    return true;
+    if (!ready) atomicOr(P.status, 1 << MCG_ERR_TIMEOUT);
 }
 
 // Fraction theta in [0, 1] of the step X -> X + dW (coordinates relative to
@@ -301,17 +252,47 @@ __device__ __forceinline__ double exit_mixed(const WalkParams& P, const ModelRef
 // 32 bytes, written as two 16-byte stores that fill one sector -- X (the walk
 // position before the exit step, copy 0's coordinates; copy c adds its z
 // offset), Y (the copy's first point not strictly inside Omega) and the
-// source sum flushed + partial in double.  rho at X is not stored:
+// source sum in double.  rho at X is not stored:
 // exit_mixed_kernel evaluates the same single-precision density function at
 // the same X, which gives the walk's value bit for bit.  The record is valid
 // once the item's step count carries kDoneFlag.
 __device__ __forceinline__ void put_exit(const WalkParams& P, int c, unsigned long long item, float x0, float x1,
-                                         float x2, float y0, float y1, float y2, float partial, double flushed)
+                                         float x2, float y0, float y1, float y2, double acc)
 {
-    const double acc = flushed + (double)partial;
     float4* r = (float4*)P.frec + 2 * ((size_t)c * P.total + item);
     r[0] = make_float4(x0, x1, x2, y0);
     r[1] = make_float4(y1, y2, __int_as_float(__double2loint(acc)), __int_as_float(__double2hiint(acc)));
+}
+
+// A density that is rho0 or 0: its source sum is rho0 times a count of
+// points, kept exactly (a single-precision count of whole and half points in
+// registers, half points as a 64-bit integer beyond it), so no double
+// precision is needed before the exit and the sum does not depend on the
+// order of its terms.
+template <int RHO>
+constexpr bool kTwoValued = RHO == MCG_RHO_PRISM || RHO == MCG_RHO_SPHERE;
+template <int RHO>
+constexpr bool kVoxel = RHO == MCG_RHO_VOXEL || RHO == kRhoVoxelPacked;
+
+// Source sum of a copy: `held` is the flushed part (a double's bits, or a
+// count of half points), `part` the single-precision part since.
+template <int RHO>
+__device__ __forceinline__ double source_sum(const WalkParams& P, unsigned long long held, float part)
+{
+    if constexpr (kTwoValued<RHO>)
+        return (double)P.rho0_f * (0.5 * (double)(long long)held + (double)part);
+    else
+        return __longlong_as_double((long long)held) + (double)part;
+}
+
+// The flushed part with `part` added.
+template <int RHO>
+__device__ __forceinline__ unsigned long long flushed(unsigned long long held, float part)
+{
+    if constexpr (kTwoValued<RHO>)
+        return held + (unsigned long long)(2.0f * part);
+    else
+        return (unsigned long long)__double_as_longlong(__longlong_as_double((long long)held) + (double)part);
 }
 
 __device__ __forceinline__ void write_path(const WalkParams& P, int32_t* status, unsigned long long item, double u0,
@@ -408,7 +389,7 @@ template <bool CRN, bool SEG>
 __global__ void __launch_bounds__(128) walk_fp64_kernel(const WalkParams P)
 {
     constexpr int NC = CRN ? 3 : 1;
-    bool busy = false, exhausted = false;
+    bool busy = false, drained = false;
     unsigned long long item = 0ull;
     uint32_t s = 0u, p = 0u;
     int64_t n = 0;
@@ -431,9 +412,11 @@ __global__ void __launch_bounds__(128) walk_fp64_kernel(const WalkParams P)
                 P.pp_steps[item] = steps;
             }
             busy = false;
-            exhausted = true;
+            drained = true;
         }
-        if (refill(P, busy, exhausted, item)) {
+        unsigned long long next = 0ull;
+        if (refill(P, busy, 32u, drained, next)) {
+            item = next;
             const double* st = P.stations;
             unsigned long long local = item, N = (unsigned long long)P.N, p0 = (unsigned long long)P.p0;
             if constexpr (SEG) {
@@ -527,19 +510,92 @@ __global__ void __launch_bounds__(128) walk_fp64_kernel(const WalkParams P)
 
 // ---------------------------------------------------------------------------
 // Mixed-precision walk: single-precision stepping and no double-precision
-// arithmetic in the step loop.  The three common-random-number copies are
-// updated branch-free; exits (rare) take a side branch that writes an exit
-// record, which exit_mixed_kernel turns into per-path values.  A warp runs up
-// to 16 blocks (64 steps) between refills, two blocks per loop iteration;
-// after them it flushes the single-precision partial sums into the double
-// sums (a real, warp-uniform branch, so the slow double-precision unit sees
-// one instruction per copy per 64 steps).  With a prism or sphere density in
-// the box, a warp whose walks all stay, by the block's radius bound, inside
-// Omega and away from the density for the next four steps only moves them
-// (one test per block instead of one per step); otherwise every step tests
-// the exit and samples the density.
-// ---------------------------------------------------------------------------
+// arithmetic in the step loop.  A warp works in one of two ways:
 //
+//  * lanes (more than kStripMax walks live): a lane steps a walk of its own;
+//    the three common-random-number copies are updated branch-free, exits
+//    (rare) take a side branch that writes an exit record, which
+//    exit_mixed_kernel turns into per-path values.  Up to 16 blocks (64
+//    steps) between refills;
+//  * strips (at most kStripMax walks live: a small launch, or the exit-time
+//    tail of a large one): k = 32 / walks lanes share a walk.  The random
+//    numbers of different blocks do not depend on one another, so each lane
+//    makes those of one block; only the positions form a serial chain, one
+//    fused multiply-add per coordinate and step, which a lane per coordinate
+//    runs through shared memory; then each lane tests and sums its own block.
+//
+// Both take the same steps in the same arithmetic, so a walk's numbers do not
+// depend on how it was run.  What bounds them, on the prism ore body (1 m
+// steps): a walk alone takes 115 ns a step as a lane (the block's dependent
+// generator, logarithm and root, ~950 cycles) and 10 ns as a strip of 32 (that
+// once per 32 blocks, and the chain, 16 cycles a block); with the GPU full,
+// lanes run 340 steps/ns, strips 240 (k = 2) to 100 (k = 32), as the chain
+// idles most lanes, so a full warp runs lanes.  Solves that this shortens:
+// 30 x 256 paths 168 -> 18 ms, 30 x 8192 paths 317 -> 155 ms.
+// ---------------------------------------------------------------------------
+constexpr unsigned kStripMax = 16;
+constexpr int kStripRow = 33;  // float4 per row: rows of one block column fall into different banks
+
+// Conservative tests of a four-step block.  No coordinate moves by more than -(nr[0] + ... + nr[5]) over the
+// block, so if that bound keeps every copy inside the conservative box
+// (ball) -- `inside` -- the block needs no exit test, and if it also stays
+// outside the density's support box -- `quiet` -- only the position changes.
+// The boxes' margin, 1e-5 of the domain, is some twenty times the
+// single-precision rounding of the bound and of the four moves.
+template <int RHO, bool BALL>
+__device__ __forceinline__ void block_bounds(const WalkParams& P, float x, float y, float z, const float nr[6],
+                                             bool& inside, bool& quiet)
+{
+    const float rs = ((nr[0] + nr[1]) + (nr[2] + nr[3])) + (nr[4] + nr[5]);  // <= 0
+    const float ax = fabsf(x) - rs, ay = fabsf(y) - rs, az = fabsf(z) - rs;
+    if (BALL) inside = fmaf(ax, ax, fmaf(ay, ay, az * az)) < P.in_r2_f;
+    else inside = ax < P.in_f[0] && ay < P.in_f[1] && az < P.in_f[2];
+    quiet = inside;
+    if constexpr (kTwoValued<RHO>)
+        quiet = inside && (fabsf(x - P.far_c[0]) + rs > P.far_h[0] || fabsf(y - P.far_c[1]) + rs > P.far_h[1] ||
+                           fabsf(z - P.far_c[2]) + rs > P.far_h[2]);
+    else if constexpr (kVoxel<RHO>)
+        quiet = false;
+}
+
+// Copies strictly inside Omega at the walk position (x, y, z): bit c for copy c.
+template <bool CRN, bool BALL>
+__device__ __forceinline__ unsigned copies_inside(const WalkParams& P, float x, float y, float z, float hf)
+{
+    unsigned ins;
+    if (BALL) {
+        // (explicit rounding: lanes and strips must take the same decisions)
+        const float q = __fmaf_rn(x, x, __fmul_rn(y, y));
+        const float zb = z + hf, zc = z - hf;
+        ins = (__fmaf_rn(z, z, q) < P.R2_f) ? 1u : 0u;
+        if (CRN) {
+            ins |= (__fmaf_rn(zb, zb, q) < P.R2_f) ? 2u : 0u;
+            ins |= (__fmaf_rn(zc, zc, q) < P.R2_f) ? 4u : 0u;
+        }
+    } else {
+        const bool inxy = fabsf(x) < P.half_f[0] && fabsf(y) < P.half_f[1];
+        ins = (inxy && fabsf(z) < P.half_f[2]) ? 1u : 0u;
+        if (CRN) {
+            ins |= (inxy && fabsf(z + hf) < P.half_f[2]) ? 2u : 0u;
+            ins |= (inxy && fabsf(z - hf) < P.half_f[2]) ? 4u : 0u;
+        }
+    }
+    return ins;
+}
+
+// Y of copy c for a bridge exit on face f below the step's end (x, y, z).
+__device__ __forceinline__ void bridge_point(const WalkParams& P, int c, int f, float x, float y, float z, float hf,
+                                             float out[3])
+{
+    out[0] = x;
+    out[1] = y;
+    out[2] = z + (c == 0 ? 0.0f : (c == 1 ? hf : -hf));
+    const float b = (f & 1) ? P.half_f[f >> 1] : -P.half_f[f >> 1];
+    if ((f >> 1) == 0) out[0] = b;
+    else if ((f >> 1) == 1) out[1] = b;
+    else out[2] = b;
+}
+
 // SEG: a multi-request launch (the segment table maps each item to its
 // request); each lane then carries its walk's generator key and model array,
 // and keeps the segment index with the walk's other cold state.
@@ -547,27 +603,32 @@ template <int RHO, bool CRN, bool BRIDGE, bool BALL, bool SEG>
 __global__ void __launch_bounds__(128, MCG_MIXED_MINB) walk_mixed_kernel(const WalkParams P)
 {
     static_assert(!(SEG && (BRIDGE || BALL)), "multi-request launches use the box without the bridge test");
+    constexpr int NC = CRN ? 3 : 1;
     // Per-walk state touched only at refills, exits and flushes lives in
     // shared memory (one slot per thread); the step loop keeps the position,
     // the partial sums, the path indices and the live-copy mask in registers.
-    __shared__ double sh_D[3][128];              // flushed sums per copy
-    __shared__ unsigned long long sh_item[128];  // work item of the walk
-    __shared__ long long sh_steps[128];          // EM steps of the copies that have exited
-    __shared__ int sh_seg[SEG ? 128 : 1];        // segment of the walk (multi-request launch)
+    __shared__ unsigned long long sh_acc[3][128];  // flushed sums per copy (source_sum)
+    __shared__ unsigned long long sh_item[128];    // work item of the walk
+    __shared__ unsigned long long sh_steps[128];   // EM steps of the copies that have exited
+    __shared__ int sh_seg[SEG ? 128 : 1];          // segment of the walk (multi-request launch)
+    // strips: the blocks' increments, then positions, then densities; the
+    // walks' positions; per copy the counts (two-valued) or the running sums
+    __shared__ float4 sh_strip[4][6 * kStripRow];
+    __shared__ float sh_base[4][3 * kStripMax];
+    using Part = std::conditional_t<kTwoValued<RHO>, unsigned, float>;  // half points, or a running sum
+    __shared__ Part sh_part[RHO == MCG_RHO_NONE ? 1 : 3][128];
+    __shared__ int sh_own[4][kStripMax];  // slot of the g-th live walk
     const int t = threadIdx.x;
-    bool busy = false, exhausted = false;
+    bool busy = false, drained = false;
     uint32_t s = 0u, p = 0u, blk = 0u;
     float wx = 0.f, wy = 0.f, wz = 0.f;
-    float S0 = 0.f, S1 = 0.f, S2 = 0.f;  // single-precision partial sums
+    float S0 = 0.f, S1 = 0.f, S2 = 0.f;  // single-precision partial sums (two-valued density: counts)
     unsigned alive = 0u;
-    const float hx = P.half_f[0], hy = P.half_f[1], hz = P.half_f[2];
     const float hf = CRN ? P.h_f : 0.0f;
     unsigned round = 0u;
     const int lane = t & 31;
     const unsigned lanes_below = (1u << lane) - 1u;
-    const bool migrate = P.pool != nullptr;
-    bool stop = false;     // cancelled: take no more work of any kind
-    bool spilled = false;  // this warp has spilled its walks once
+    bool stop = false;  // cancelled: take no more work of any kind
     uint32_t k0 = P.key0, k1 = P.key1;  // generator key of the lane's walk
     ModelRef M = model_of(P);           // model arrays of the lane's walk
     // the lane's walk now belongs to the request of launch item `it`
@@ -581,21 +642,32 @@ __global__ void __launch_bounds__(128, MCG_MIXED_MINB) walk_mixed_kernel(const W
             sh_seg[t] = gi;
         }
     };
+    auto flush = [&]() {
+        if constexpr (RHO != MCG_RHO_NONE) {
+            sh_acc[0][t] = flushed<RHO>(sh_acc[0][t], S0);
+            S0 = 0.f;
+            if (CRN) {
+                sh_acc[1][t] = flushed<RHO>(sh_acc[1][t], S1);
+                sh_acc[2][t] = flushed<RHO>(sh_acc[2][t], S2);
+                S1 = S2 = 0.f;
+            }
+        }
+    };
 
     for (;;) {
         if ((++round & 15u) == 0u && cancelled(P)) {
-            // walks in flight, pooled walks and unclaimed items give no result
+            // walks in flight and unclaimed items give no result
             if (lane == 0) atomicOr(P.status, 1 << MCG_ERR_CANCELLED);
             if (busy) {
                 const unsigned long long it = sh_item[t];  // (no completion flag: NaN)
-                P.pp_steps[it] = sh_steps[t] + (long long)__popc(alive) * 4 * (long long)blk;
+                P.pp_steps[it] = (long long)sh_steps[t] + (long long)__popc(alive) * 4 * (long long)blk;
             }
             busy = false;
-            exhausted = true;
+            drained = true;
             stop = true;
         }
         unsigned long long item = 0ull;
-        bool start = refill(P, busy, exhausted, item);
+        bool start = refill(P, busy, (unsigned)P.quota, drained, item);
         const double* st = P.stations;
         if (start) {
             unsigned long long local = item, N = (unsigned long long)P.N, p0 = (unsigned long long)P.p0;
@@ -617,100 +689,341 @@ __global__ void __launch_bounds__(128, MCG_MIXED_MINB) walk_mixed_kernel(const W
             wx = (float)(st[3 * s + 0] - P.cen[0]);
             wy = (float)(st[3 * s + 1] - P.cen[1]);
             wz = (float)(st[3 * s + 2] - P.cen[2]);
-            float r0, r1, r2;
-            rho3_f32<RHO>(P, SEG ? M : model_of(P), wx, wy, wz, hf, r0, r1, r2);
-            S0 = 0.5f * r0;
-            S1 = 0.5f * r1;
-            S2 = 0.5f * r2;
-            sh_D[0][t] = sh_D[1][t] = sh_D[2][t] = 0.0;
+            if constexpr (kTwoValued<RHO>) {
+                const unsigned in = support3_f32<RHO>(P, wx, wy, wz, hf);
+                S0 = (in & 1u) ? 0.5f : 0.0f;
+                S1 = (in & 2u) ? 0.5f : 0.0f;
+                S2 = (in & 4u) ? 0.5f : 0.0f;
+            } else {
+                float r0, r1, r2;
+                rho3_f32<RHO>(P, SEG ? M : model_of(P), wx, wy, wz, hf, r0, r1, r2);
+                S0 = 0.5f * r0;
+                S1 = 0.5f * r1;
+                S2 = 0.5f * r2;
+            }
+            sh_acc[0][t] = sh_acc[1][t] = sh_acc[2][t] = 0ull;
             sh_item[t] = item;
-            sh_steps[t] = 0;
+            sh_steps[t] = 0ull;
             alive = CRN ? 7u : 1u;
             blk = 0u;
             busy = true;
         }
-        if (migrate && !stop) {
-            // the work list is used up: fill free lanes with pooled walks
-            const unsigned freem = __ballot_sync(kFull, !busy);
-            if (freem && __any_sync(kFull, exhausted)) {
-                unsigned long long base = 0ull;
-                unsigned got = 0u;
-                if (lane == 0) got = pool_take(P, (unsigned)__popc(freem), base);
-                got = __shfl_sync(kFull, got, 0);
-                base = __shfl_sync(kFull, base, 0);
-                const unsigned rank = (unsigned)__popc(freem & lanes_below);
-                if (!busy && rank < got) {
-                    const unsigned long long slot = base + rank;
-                    uint32_t ready = 0u;
-                    for (int i = 0; i < kReadySpin && !ready; ++i) {
-                        ready = ld_acquire_u32(P.pool_ready + slot);
-                        if (!ready) __nanosleep(64);
-                    }
-                    if (ready) {
-                        const uint4* e = (const uint4*)(P.pool + slot * kPoolEntryBytes);
-                        const uint4 e0 = e[0], e1 = e[1], e2 = e[2], e3 = e[3], e4 = e[4];
-                        sh_item[t] = ((unsigned long long)e0.y << 32) | e0.x;
-                        adopt(sh_item[t]);
-                        blk = e0.z;
-                        alive = e0.w;
-                        wx = __uint_as_float(e1.x);
-                        wy = __uint_as_float(e1.y);
-                        wz = __uint_as_float(e1.z);
-                        s = e1.w;
-                        p = e2.x;
-                        sh_steps[t] = (long long)(((unsigned long long)e2.w << 32) | e2.z);
-                        sh_D[0][t] = __hiloint2double((int)e3.y, (int)e3.x);
-                        sh_D[1][t] = __hiloint2double((int)e3.w, (int)e3.z);
-                        sh_D[2][t] = __hiloint2double((int)e4.y, (int)e4.x);
-                        S0 = S1 = S2 = 0.f;
-                        busy = true;
-                    } else {
-                        atomicOr(P.status, 1 << MCG_ERR_TIMEOUT);
-                    }
-                }
-            }
-        }
-        unsigned livem = __ballot_sync(kFull, busy);
-        if (migrate && !stop && !spilled && livem != 0u && __popc(livem) <= P.spill_max &&
-            __any_sync(kFull, exhausted)) {
-            // few walks left here and nothing new to start: hand them over
-            unsigned long long base = 0ull;
-            int ok = 0;
-            if (lane == 0) ok = pool_reserve(P, (unsigned)__popc(livem), base) ? 1 : 0;
-            if (__shfl_sync(kFull, ok, 0)) {
-                base = __shfl_sync(kFull, base, 0);
-                if (busy) {
-                    const unsigned long long slot = base + (unsigned)__popc(livem & lanes_below);
-                    const unsigned long long it = sh_item[t];
-                    const unsigned long long st = (unsigned long long)sh_steps[t];
-                    const double D0 = sh_D[0][t] + (double)S0, D1 = sh_D[1][t] + (double)S1,
-                                 D2 = sh_D[2][t] + (double)S2;
-                    uint4* e = (uint4*)(P.pool + slot * kPoolEntryBytes);
-                    e[0] = make_uint4((uint32_t)it, (uint32_t)(it >> 32), blk, alive);
-                    e[1] = make_uint4(__float_as_uint(wx), __float_as_uint(wy), __float_as_uint(wz), s);
-                    e[2] = make_uint4(p, 0u, (uint32_t)st, (uint32_t)(st >> 32));
-                    e[3] = make_uint4((uint32_t)__double2loint(D0), (uint32_t)__double2hiint(D0),
-                                      (uint32_t)__double2loint(D1), (uint32_t)__double2hiint(D1));
-                    e[4] = make_uint4((uint32_t)__double2loint(D2), (uint32_t)__double2hiint(D2), 0u, 0u);
-                    st_release_u32(P.pool_ready + slot, 1u);
-                    busy = false;
-                }
-                spilled = true;
-                livem = 0u;
-            }
-        }
+        const unsigned livem = __ballot_sync(kFull, busy);
         if (livem == 0u) {
-            if (!migrate) break;
-            int leave = 1;
-            if (lane == 0) leave = pool_leave(P, stop) ? 1 : 0;
-            if (__shfl_sync(kFull, leave, 0)) break;
-            continue;  // the last warp: take over the pooled walks
+            if (!drained) continue;  // (every claimed station lay outside Omega)
+            if (P.fault_unpublished && P.pool && !stop && lane == 0) pool_wait(P);
+            break;
+        }
+
+        if (__popc(livem) <= (int)kStripMax) {
+            // ----------------------------------------------------------------
+            // Strips.  Group g of k lanes runs the g-th live walk; what the
+            // group's lanes share is held alike in all of them.
+            // ----------------------------------------------------------------
+            const int G = __popc(livem), k = 32 / G;
+            const int g = lane / k < G ? lane / k : G - 1;
+            const bool mine = lane / k < G;          // this lane belongs to a group
+            const int l = lane - g * k;              // its block of the group's round
+            float4* strip = sh_strip[t >> 5];
+            float* base = sh_base[t >> 5];
+            const int* own = sh_own[t >> 5];
+            const int rank = __popc(livem & lanes_below);
+            // the counts move as half points, the running sums as they are
+            auto part_of = [](float v) -> Part { return kTwoValued<RHO> ? (Part)(2.0f * v) : (Part)v; };
+            auto value_of = [](Part v) -> float { return kTwoValued<RHO> ? 0.5f * (float)v : (float)v; };
+            if (busy) {
+                sh_own[t >> 5][rank] = t;
+                base[3 * rank] = wx;
+                base[3 * rank + 1] = wy;
+                base[3 * rank + 2] = wz;
+                if constexpr (RHO != MCG_RHO_NONE) {
+                    sh_part[0][t] = part_of(S0);
+                    if (CRN) {
+                        sh_part[1][t] = part_of(S1);
+                        sh_part[2][t] = part_of(S2);
+                    }
+                }
+            }
+            __syncwarp();
+            const int slot = own[g], owner = slot & 31;
+            const unsigned gmask = (k == 32 ? kFull : ((1u << k) - 1u)) << (g * k);
+            const uint32_t gs = __shfl_sync(kFull, s, owner), gp = __shfl_sync(kFull, p, owner);
+            uint32_t gblk = __shfl_sync(kFull, blk, owner);
+            unsigned gal = __shfl_sync(kFull, alive, owner);
+            uint32_t gk0 = k0, gk1 = k1;
+            ModelRef gM = M;
+            if constexpr (SEG) {
+                gk0 = __shfl_sync(kFull, k0, owner);
+                gk1 = __shfl_sync(kFull, k1, owner);
+                gM.grid = (const float*)__shfl_sync(kFull, (unsigned long long)M.grid, owner);
+                gM.zq = (const float4*)__shfl_sync(kFull, (unsigned long long)M.zq, owner);
+            }
+            unsigned N0 = 0u, N1 = 0u, N2 = 0u;  // this lane's points of the support, not yet in sh_part
+            auto add_counts = [&]() {
+                if (N0) atomicAdd((unsigned*)&sh_part[0][slot], 2u * N0);
+                if (CRN && N1) atomicAdd((unsigned*)&sh_part[1][slot], 2u * N1);
+                if (CRN && N2) atomicAdd((unsigned*)&sh_part[2][slot], 2u * N2);
+                N0 = N1 = N2 = 0u;
+                __syncwarp();
+            };
+            // the block at whose end a live walk has reached the step cap
+            const int64_t cap_blk = (P.max_steps + 3) / 4;
+            bool ended = false;  // the group's walk is complete or capped
+            for (int r = 0; r < 16; ++r) {
+                // blocks of this round: up to k, not past the cap, and for a
+                // density that is summed in single precision not past the
+                // next flush (every 16 blocks)
+                int kk = k;
+                if constexpr (kVoxel<RHO>) kk = min(kk, 16 - (int)(gblk & 15u));
+                if ((int64_t)gblk + kk > cap_blk) kk = (int)(cap_blk - (int64_t)gblk);
+                const bool act = mine && l < kk;
+                float nr[6], cs[12];
+                polar12_f32(gs, gp, gblk + (uint32_t)l, SEG ? gk0 : P.key0, SEG ? gk1 : P.key1, P.lnscale_f, nr, cs);
+                // the moves per coordinate, four steps to a float4: radii in
+                // rows 0-2, cosines or sines in rows 3-5
+                strip[0 * kStripRow + lane] = make_float4(nr[0], nr[1], nr[3], nr[4]);
+                strip[1 * kStripRow + lane] = make_float4(nr[0], nr[2], nr[3], nr[5]);
+                strip[2 * kStripRow + lane] = make_float4(nr[1], nr[2], nr[4], nr[5]);
+                strip[3 * kStripRow + lane] = make_float4(cs[0], cs[3], cs[6], cs[9]);
+                strip[4 * kStripRow + lane] = make_float4(cs[1], cs[4], cs[7], cs[10]);
+                strip[5 * kStripRow + lane] = make_float4(cs[2], cs[5], cs[8], cs[11]);
+                __syncwarp();
+                float4 w0 = make_float4(base[3 * g], base[3 * g + 1], base[3 * g + 2], 0.f);  // before the round
+                // the chain of positions: lane q runs coordinate q % 3 of walk
+                // q / 3 and leaves the four positions of each block in rows 0-2
+                for (int q = lane; q < 3 * G; q += 32) {
+                    float x = base[q];
+                    float4* rr = strip + (q % 3) * kStripRow + (q / 3) * k;
+                    const float4* cc = rr + 3 * kStripRow;
+                    auto four = [&x](const float4& a, const float4& b) {
+                        float4 y;
+                        x = y.x = fmaf(a.x, b.x, x);
+                        x = y.y = fmaf(a.y, b.y, x);
+                        x = y.z = fmaf(a.z, b.z, x);
+                        x = y.w = fmaf(a.w, b.w, x);
+                        return y;
+                    };
+                    // two blocks at a time, the next two loaded meanwhile
+                    // (32 cycles of arithmetic cover a shared-memory read)
+                    float4 a0 = rr[0], b0 = cc[0], a1 = rr[1], b1 = cc[1];  // k >= 2
+                    int i = 0;
+                    for (; i + 4 <= k; i += 2) {
+                        const float4 a2 = rr[i + 2], b2 = cc[i + 2], a3 = rr[i + 3], b3 = cc[i + 3];
+                        rr[i] = four(a0, b0);
+                        rr[i + 1] = four(a1, b1);
+                        a0 = a2;
+                        b0 = b2;
+                        a1 = a3;
+                        b1 = b3;
+                    }
+                    rr[i] = four(a0, b0);
+                    rr[i + 1] = four(a1, b1);
+                    if (i + 2 < k) rr[i + 2] = four(rr[i + 2], cc[i + 2]);  // k odd
+                }
+                __syncwarp();
+                const float4 X = strip[0 * kStripRow + lane], Y = strip[1 * kStripRow + lane],
+                             Z = strip[2 * kStripRow + lane];
+                {   // the position before this lane's block
+                    const float x = __shfl_up_sync(kFull, X.w, 1), y = __shfl_up_sync(kFull, Y.w, 1),
+                                z = __shfl_up_sync(kFull, Z.w, 1);
+                    if (l > 0) {
+                        w0.x = x;
+                        w0.y = y;
+                        w0.z = z;
+                    }
+                }
+                __syncwarp();
+                if (act && l == kk - 1) {
+                    base[3 * g] = X.w;
+                    base[3 * g + 1] = Y.w;
+                    base[3 * g + 2] = Z.w;
+                }
+                bool inside, quiet;
+                block_bounds<RHO, BALL>(P, w0.x, w0.y, w0.z, nr, inside, quiet);
+                const bool all_inside = __all_sync(kFull, inside || !act);
+                const bool all_quiet = __all_sync(kFull, quiet || !act);
+                if (!all_quiet) {
+                    const float px[5] = {w0.x, X.x, X.y, X.z, X.w}, py[5] = {w0.y, Y.x, Y.y, Y.z, Y.w},
+                                pz[5] = {w0.z, Z.x, Z.y, Z.z, Z.w};
+                    const uint32_t myblk = gblk + (uint32_t)l;
+                    unsigned la = act ? gal : 0u;  // copies live at this point of the block
+                    unsigned out = 0u;             // copies that leave in this block ...
+                    unsigned om = 0u, of = 0u;     // ... their step (2 bits each); bridge face + 1 (3 bits each)
+                    unsigned n0 = 0u, n1 = 0u, n2 = 0u;  // points of the density's support (two-valued)
+                    float rv[4][3];
+#pragma unroll
+                    for (int m = 0; m < 4; ++m) {
+                        if (!all_inside) {
+                            const unsigned ins = copies_inside<CRN, BALL>(P, px[m + 1], py[m + 1], pz[m + 1], hf);
+                            const unsigned gone = la & ~ins;
+                            if (gone) {
+                                out |= gone;
+#pragma unroll
+                                for (int c = 0; c < NC; ++c)
+                                    if (gone & (1u << c)) om |= (unsigned)m << (2 * c);
+                                la &= ins;
+                            }
+                            if (BRIDGE && la) {
+                                unsigned faces = 0u;
+                                const unsigned bx = bridge_exits_f32(P, la, px[m], py[m], pz[m], px[m + 1], py[m + 1],
+                                                                     pz[m + 1], hf, gs, gp, myblk, m, &faces);
+                                if (bx) {
+                                    out |= bx;
+                                    la &= ~bx;
+#pragma unroll
+                                    for (int c = 0; c < NC; ++c)
+                                        if (bx & (1u << c)) {
+                                            om |= (unsigned)m << (2 * c);
+                                            of |= (((faces >> (3 * c)) & 7u) + 1u) << (3 * c);
+                                        }
+                                }
+                            }
+                        }
+                        if constexpr (kTwoValued<RHO>) {
+                            const unsigned in = la & support3_f32<RHO>(P, px[m + 1], py[m + 1], pz[m + 1], hf);
+                            n0 += in & 1u;
+                            n1 += (in >> 1) & 1u;
+                            n2 += in >> 2;
+                        } else if constexpr (kVoxel<RHO>) {
+                            rho3_f32<RHO>(P, SEG ? gM : model_of(P), px[m + 1], py[m + 1], pz[m + 1], hf, rv[m][0],
+                                          rv[m][1], rv[m][2]);
+                        }
+                    }
+                    // the first block of the round in which each copy leaves
+                    int first[3] = {32, 32, 32};
+                    const bool any_out = __any_sync(kFull, out != 0u);
+                    if (any_out) {
+#pragma unroll
+                        for (int c = 0; c < NC; ++c) {
+                            const unsigned b = __ballot_sync(kFull, (out >> c) & 1u) & gmask;
+                            if (b) first[c] = __ffs(b) - 1;
+                        }
+                    }
+                    float pre[3] = {0.f, 0.f, 0.f};  // single-precision sums before this block (voxel)
+                    if constexpr (kTwoValued<RHO>) {
+                        // counts up to the exit; exact, so the order does not matter
+                        if (lane <= first[0]) N0 += n0;
+                        if (CRN && lane <= first[1]) N1 += n1;
+                        if (CRN && lane <= first[2]) N2 += n2;
+                        if (any_out) add_counts();
+                    } else if constexpr (kVoxel<RHO>) {
+                        // the same order of additions as a lane's: a chain
+                        // over the round's blocks, lane q copy q % NC of walk q / NC
+#pragma unroll
+                        for (int c = 0; c < NC; ++c)
+                            strip[(3 + c) * kStripRow + lane] =
+                                act ? make_float4(rv[0][c], rv[1][c], rv[2][c], rv[3][c]) : make_float4(0.f, 0.f, 0.f, 0.f);
+                        __syncwarp();
+                        for (int q = lane; q < NC * G; q += 32) {
+                            const int gq = q / NC, c = q % NC;
+                            Part* part = &sh_part[c][own[gq]];
+                            float S = value_of(*part);
+                            float4* rr = strip + c * kStripRow + gq * k;
+                            for (int i = 0; i < k; ++i) {
+                                const float4 v = rr[3 * kStripRow + i];
+                                rr[i].x = S;
+                                S += v.x;
+                                S += v.y;
+                                S += v.z;
+                                S += v.w;
+                            }
+                            *part = part_of(S);
+                        }
+                        __syncwarp();
+#pragma unroll
+                        for (int c = 0; c < NC; ++c) pre[c] = strip[c * kStripRow + lane].x;
+                    }
+                    if (any_out) {
+                        const unsigned left = (first[0] < 32 ? 1u : 0u) | (first[1] < 32 ? 2u : 0u) |
+                                              (first[2] < 32 ? 4u : 0u);
+#pragma unroll
+                        for (int c = 0; c < NC; ++c) {
+                            if (!mine || lane != first[c]) continue;
+                            const unsigned m = (om >> (2 * c)) & 3u;
+                            float x = 0.f, y = 0.f, z = 0.f, e[3] = {0.f, 0.f, 0.f}, ez = 0.f;
+                            float part = pre[c];
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) {
+                                if (i == (int)m) {
+                                    x = px[i];
+                                    y = py[i];
+                                    z = pz[i];
+                                    e[0] = px[i + 1];
+                                    e[1] = py[i + 1];
+                                    ez = pz[i + 1];
+                                }
+                                if constexpr (kVoxel<RHO>)
+                                    if (i < (int)m) part += rv[i][c];
+                            }
+                            if constexpr (kTwoValued<RHO>) part = value_of(sh_part[c][slot]);
+                            e[2] = c == 0 ? ez : (c == 1 ? ez + hf : ez - hf);
+                            if constexpr (BRIDGE) {
+                                const int f = (int)((of >> (3 * c)) & 7u) - 1;
+                                if (f >= 0) bridge_point(P, c, f, e[0], e[1], ez, hf, e);
+                            }
+                            put_exit(P, c, sh_item[slot], x, y, z, e[0], e[1], e[2],
+                                     RHO == MCG_RHO_NONE ? 0.0 : source_sum<RHO>(P, sh_acc[c][slot], part));
+                            atomicAdd(&sh_steps[slot], (unsigned long long)nstep_of(myblk, (int)m));
+                        }
+                        gal &= ~left;
+                        __syncwarp();
+                    }
+                }
+                gblk += (uint32_t)kk;
+                if constexpr (kVoxel<RHO>) {
+                    if ((gblk & 15u) == 0u && l < NC && mine) {  // flush (k >= 2: two lanes may take three copies)
+                        for (int c = l; c < NC; c += k) {
+                            sh_acc[c][slot] = flushed<RHO>(sh_acc[c][slot], value_of(sh_part[c][slot]));
+                            sh_part[c][slot] = (Part)0;
+                        }
+                    }
+                }
+                if (mine && gal == 0u) {
+                    if (l == 0) P.pp_steps[sh_item[slot]] = (long long)(sh_steps[slot] | (unsigned long long)kDoneFlag);
+                    ended = true;
+                } else if (mine && (int64_t)gblk >= cap_blk) {
+                    if (l == 0) {
+                        atomicOr(SEG ? P.seg[sh_seg[slot]].status : P.status, 1 << MCG_ERR_STEP_CAP);
+                        // (no completion flag: the exit kernel writes NaN)
+                        P.pp_steps[sh_item[slot]] =
+                            (long long)sh_steps[slot] + (long long)__popc(gal) * 4 * (long long)gblk;
+                    }
+                    ended = true;
+                }
+                __syncwarp();
+                if (__any_sync(kFull, ended)) break;  // regroup the others, or take new walks
+            }
+            // back to the owners
+            if constexpr (kTwoValued<RHO>) add_counts();
+            const int from = rank * k & 31;
+            const uint32_t nb = __shfl_sync(kFull, gblk, from);
+            const unsigned na = __shfl_sync(kFull, gal, from);
+            const int ne = __shfl_sync(kFull, (int)ended, from);
+            if (busy) {
+                wx = base[3 * rank];
+                wy = base[3 * rank + 1];
+                wz = base[3 * rank + 2];
+                blk = nb;
+                alive = na;
+                if constexpr (RHO != MCG_RHO_NONE) {
+                    S0 = value_of(sh_part[0][t]);
+                    if (CRN) {
+                        S1 = value_of(sh_part[1][t]);
+                        S2 = value_of(sh_part[2][t]);
+                    }
+                }
+                if (ne) busy = false;
+            }
+            __syncwarp();
+            if constexpr (kTwoValued<RHO>)
+                if ((round & 63u) == 0u) flush();  // counts stay below 2^22 (at most 2048 steps a round)
+            continue;
         }
 
         // two four-step blocks per iteration for the analytic densities; one
         // for the voxel grid, whose larger step body (prefetched lookups)
         // otherwise strains the instruction cache
-        constexpr int kBlocksUnrolled = (RHO == MCG_RHO_VOXEL || RHO == kRhoVoxelPacked) ? 1 : 2;
+        constexpr int kBlocksUnrolled = kVoxel<RHO> ? 1 : 2;
 #pragma unroll (kBlocksUnrolled)
         for (int k = 0; k < 16; ++k) {
             if (busy) {
@@ -722,67 +1035,26 @@ __global__ void __launch_bounds__(128, MCG_MIXED_MINB) walk_mixed_kernel(const W
                 polar12_f32(s, p, blk, SEG ? k0 : P.key0, SEG ? k1 : P.key1, P.lnscale_f, nr, cs);
                 // one fused multiply-add per coordinate and step
                 auto mv = [&](float x, int j) -> float { return fmaf(nr[j >> 1], cs[j], x); };
+                // The block tests are taken for the warp (all live lanes), so
+                // a warp never runs both the quiet moves and the full steps.
+                // (Not for the voxel grid: the second copy of the step body
+                // costs its kernel six registers and a sixth of its resident
+                // warps.)
+                constexpr bool kBlockTest = !kVoxel<RHO>;
+                bool all_quiet = false, all_inside = false;
+                if constexpr (kBlockTest) {
+                    bool inside, quiet;
+                    block_bounds<RHO, BALL>(P, wx, wy, wz, nr, inside, quiet);
+                    const unsigned am = __activemask();
+                    all_quiet = __all_sync(am, quiet);
+                    all_inside = __all_sync(am, inside);
+                }
                 // Voxel grid: the block's four positions are known once its
                 // normals are, so all twelve density loads are issued here
                 // and their latency overlaps the steps (same positions, same
                 // summation order: results are unchanged).
-                constexpr bool kPrefetch = RHO == MCG_RHO_VOXEL || RHO == kRhoVoxelPacked;
-                // Quiet block (box domain, prism or sphere density): no
-                // coordinate moves by more than -(nr[0] + ... + nr[5]) over
-                // the block, so if that bound keeps every copy inside the
-                // conservative box and outside the density's support box for
-                // the whole block, the four steps only move (the boxes' margin,
-                // 1e-5 of the domain, is some twenty times the single-precision
-                // rounding of the bound and of the four moves).  The decision is
-                // taken for the warp (all live lanes quiet), so a warp never
-                // runs both the quiet moves and the full steps.
-                constexpr bool kBlockTest = !BALL && !kPrefetch &&
-                                            (RHO == MCG_RHO_PRISM || RHO == MCG_RHO_SPHERE);
-                // The same bound with the domain alone: a warp whose copies all
-                // stay surely inside Omega for the block runs its steps without
-                // exit tests.  (Not for the voxel grid: the second copy of the
-                // step body costs its kernel six registers and a sixth of its
-                // resident warps.)
-                constexpr bool kBlockInside = !BALL && !kPrefetch;
-                bool all_quiet = false, all_inside = false;
-                if constexpr (kBlockTest || kBlockInside) {
-                    const float rs = ((nr[0] + nr[1]) + (nr[2] + nr[3])) + (nr[4] + nr[5]);  // <= 0
-                    const bool inside =
-                        fabsf(wx) - rs < P.in_f[0] && fabsf(wy) - rs < P.in_f[1] && fabsf(wz) - rs < P.in_f[2];
-                    const unsigned am = __activemask();
-                    if constexpr (kBlockTest) {
-                        const bool far = fabsf(wx - P.far_c[0]) + rs > P.far_h[0] ||
-                                         fabsf(wy - P.far_c[1]) + rs > P.far_h[1] ||
-                                         fabsf(wz - P.far_c[2]) + rs > P.far_h[2];
-                        all_quiet = __all_sync(am, inside && far);
-                    }
-                    if constexpr (kBlockInside) all_inside = __all_sync(am, inside);
-                }
-                // common step: every copy surely inside Omega and surely
-                // outside the density's support -> nothing to do but move
-                // (ki: the block test already showed every copy inside)
-                auto common = [&](auto ki, float nx, float ny, float nz, bool& inside_all, float& qxy) -> bool {
-                    qxy = BALL ? nx * nx + ny * ny : 0.0f;
-                    if constexpr (decltype(ki)::value)
-                        inside_all = true;
-                    else
-                        inside_all = BALL ? qxy + nz * nz < P.in_r2_f
-                                          : fabsf(nx) < P.in_f[0] && fabsf(ny) < P.in_f[1] && fabsf(nz) < P.in_f[2];
-                    if constexpr (kBlockTest) return false;  // the block test decided: full step
-                    bool no_rho = true;
-                    if constexpr (RHO == MCG_RHO_PRISM) {
-                        no_rho = !(fabsf(nx - P.far_c[0]) <= P.far_h[0] && fabsf(ny - P.far_c[1]) <= P.far_h[1] &&
-                                   fabsf(nz - P.far_c[2]) <= P.far_h[2]);
-                    } else if constexpr (RHO == MCG_RHO_SPHERE) {
-                        const float dx = nx - P.sc_f[0], dy = ny - P.sc_f[1], dz = nz - P.sc_f[2];
-                        no_rho = dx * dx + dy * dy + dz * dz > P.far_r2;
-                    } else if constexpr (RHO == MCG_RHO_VOXEL || RHO == kRhoVoxelPacked) {
-                        no_rho = false;
-                    }
-                    return inside_all && no_rho;
-                };
                 float px[4], py[4], pz[4], rv[4][3];
-                if constexpr (kPrefetch) {
+                if constexpr (kVoxel<RHO>) {
                     float x = wx, y = wy, zz = wz;
 #pragma unroll
                     for (int m = 0; m < 4; ++m) {
@@ -806,84 +1078,59 @@ __global__ void __launch_bounds__(128, MCG_MIXED_MINB) walk_mixed_kernel(const W
                     auto full_steps = [&](auto ki) {
 #pragma unroll
                     for (int m = 0; m < 4; ++m) {
-                        const float nx = kPrefetch ? px[m] : mv(wx, 3 * m);
-                        const float ny = kPrefetch ? py[m] : mv(wy, 3 * m + 1);
-                        const float nz = kPrefetch ? pz[m] : mv(wz, 3 * m + 2);
-                        bool inside_all;
-                        float qxy;
-                        if (!common(ki, nx, ny, nz, inside_all, qxy)) {  // otherwise rho = 0 at every copy: sums unchanged
-                            if (!inside_all) {
-                                unsigned ins;
-                                if (BALL) {
-                                    const float za = nz, zb = nz + hf, zc = nz - hf;
-                                    ins = (qxy + za * za < P.R2_f) ? 1u : 0u;
-                                    if (CRN) {
-                                        ins |= (qxy + zb * zb < P.R2_f) ? 2u : 0u;
-                                        ins |= (qxy + zc * zc < P.R2_f) ? 4u : 0u;
-                                    }
-                                } else {
-                                    const bool inxy = fabsf(nx) < hx && fabsf(ny) < hy;
-                                    ins = (inxy && fabsf(nz) < hz) ? 1u : 0u;
-                                    if (CRN) {
-                                        ins |= (inxy && fabsf(nz + hf) < hz) ? 2u : 0u;
-                                        ins |= (inxy && fabsf(nz - hf) < hz) ? 4u : 0u;
-                                    }
-                                }
-                                const unsigned out = alive & ~ins;
-                                if (out) {  // some copy left Omega on this step
+                        const float nx = kVoxel<RHO> ? px[m] : mv(wx, 3 * m);
+                        const float ny = kVoxel<RHO> ? py[m] : mv(wy, 3 * m + 1);
+                        const float nz = kVoxel<RHO> ? pz[m] : mv(wz, 3 * m + 2);
+                        // surely inside: by the block test, or (voxel grid) by a test of the step
+                        bool inside_all = decltype(ki)::value;
+                        if constexpr (!kBlockTest && !decltype(ki)::value)
+                            inside_all = fabsf(nx) < P.in_f[0] && fabsf(ny) < P.in_f[1] && fabsf(nz) < P.in_f[2];
+                        if (!inside_all) {
+                            const unsigned ins = copies_inside<CRN, BALL>(P, nx, ny, nz, hf);
+                            const unsigned out = alive & ~ins;
+                            if (out) {  // some copy left Omega on this step
+                                const unsigned long long it = sh_item[t];
+                                auto sum = [&](int c, float part) {
+                                    return RHO == MCG_RHO_NONE ? 0.0 : source_sum<RHO>(P, sh_acc[c][t], part);
+                                };
+                                if (out & 1u) put_exit(P, 0, it, wx, wy, wz, nx, ny, nz, sum(0, S0));
+                                if (CRN && (out & 2u)) put_exit(P, 1, it, wx, wy, wz, nx, ny, nz + hf, sum(1, S1));
+                                if (CRN && (out & 4u)) put_exit(P, 2, it, wx, wy, wz, nx, ny, nz - hf, sum(2, S2));
+                                sh_steps[t] += (unsigned long long)nstep_of(blk, m) * __popc(out);
+                                alive &= ins;
+                            }
+                            if (BRIDGE && alive) {  // within the bridge band of a face
+                                unsigned faces = 0u;
+                                const unsigned bx = bridge_exits_f32(P, alive, wx, wy, wz, nx, ny, nz, hf, s, p, blk, m,
+                                                                     &faces);
+                                if (bx) {
                                     const unsigned long long it = sh_item[t];
-                                    if (out & 1u) put_exit(P, 0, it, wx, wy, wz, nx, ny, nz, S0, sh_D[0][t]);
-                                    if (CRN && (out & 2u)) put_exit(P, 1, it, wx, wy, wz, nx, ny, nz + hf, S1, sh_D[1][t]);
-                                    if (CRN && (out & 4u)) put_exit(P, 2, it, wx, wy, wz, nx, ny, nz - hf, S2, sh_D[2][t]);
-                                    sh_steps[t] += nstep_of(blk, m) * (long long)__popc(out);
-                                    alive &= ins;
-                                }
-                                if (BRIDGE && alive) {  // within the bridge band of a face
-                                    unsigned faces = 0u;
-                                    const unsigned bx = bridge_exits_f32(P, alive, wx, wy, wz, nx, ny, nz, hf, s, p, blk, m,
-                                                                         &faces);
-                                    if (bx) {
-                                        const unsigned long long it = sh_item[t];
-                                        const float yb[3] = {nx, ny, nz};
-                                        for (int c = 0; c < 3; ++c) {
-                                            if (!(bx & (1u << c))) continue;
-                                            const float off = c == 0 ? 0.0f : (c == 1 ? hf : -hf);
-                                            float y3[3] = {yb[0], yb[1], yb[2] + off};
-                                            const int f = (int)((faces >> (3 * c)) & 7u);
-                                            y3[f >> 1] = (f & 1) ? P.half_f[f >> 1] : -P.half_f[f >> 1];
-                                            const float part = c == 0 ? S0 : (c == 1 ? S1 : S2);
-                                            put_exit(P, c, it, wx, wy, wz, y3[0], y3[1], y3[2], part, sh_D[c][t]);
-                                        }
-                                        sh_steps[t] += nstep_of(blk, m) * (long long)__popc(bx);
-                                        alive &= ~bx;
+                                    for (int c = 0; c < 3; ++c) {
+                                        if (!(bx & (1u << c))) continue;
+                                        float e[3];
+                                        bridge_point(P, c, (int)((faces >> (3 * c)) & 7u), nx, ny, nz, hf, e);
+                                        const float part = c == 0 ? S0 : (c == 1 ? S1 : S2);
+                                        put_exit(P, c, it, wx, wy, wz, e[0], e[1], e[2],
+                                                 RHO == MCG_RHO_NONE ? 0.0 : source_sum<RHO>(P, sh_acc[c][t], part));
                                     }
+                                    sh_steps[t] += (unsigned long long)nstep_of(blk, m) * __popc(bx);
+                                    alive &= ~bx;
                                 }
                             }
-                            if constexpr (RHO == MCG_RHO_PRISM) {
-                                // the prism's density is rho0 or 0: add rho0 where a
-                                // copy is inside (the tests of rho3_f32<PRISM>)
-                                const bool inxy = nx >= P.plo_f[0] && nx < P.phi_f[0] && ny >= P.plo_f[1] &&
-                                                  ny < P.phi_f[1];
-                                const float zb = __fadd_rn(nz, hf), zc = __fsub_rn(nz, hf);
-                                if (inxy && nz >= P.plo_f[2] && nz < P.phi_f[2]) S0 += P.rho0_f;
-                                if (CRN) {
-                                    if (inxy && zb >= P.plo_f[2] && zb < P.phi_f[2]) S1 += P.rho0_f;
-                                    if (inxy && zc >= P.plo_f[2] && zc < P.phi_f[2]) S2 += P.rho0_f;
-                                }
-                            } else {
-                                float ra, rb, rc;
-                                if constexpr (kPrefetch) {
-                                    ra = rv[m][0];
-                                    rb = rv[m][1];
-                                    rc = rv[m][2];
-                                } else {
-                                    rho3_f32<RHO>(P, SEG ? M : model_of(P), nx, ny, nz, hf, ra, rb, rc);
-                                }
-                                S0 += ra;
-                                if (CRN) {
-                                    S1 += rb;
-                                    S2 += rc;
-                                }
+                        }
+                        if constexpr (kTwoValued<RHO>) {
+                            // count where a copy is in the density's support
+                            // (no live-copy test: a copy that has left has
+                            // its record, its count is not read again)
+                            const unsigned in = support3_f32<RHO>(P, nx, ny, nz, hf);
+                            if (in & 1u) S0 += 1.0f;
+                            if (CRN && (in & 2u)) S1 += 1.0f;
+                            if (CRN && (in & 4u)) S2 += 1.0f;
+                        } else if constexpr (kVoxel<RHO>) {
+                            S0 += rv[m][0];
+                            if (CRN) {
+                                S1 += rv[m][1];
+                                S2 += rv[m][2];
                             }
                         }
                         wx = nx;
@@ -894,34 +1141,29 @@ __global__ void __launch_bounds__(128, MCG_MIXED_MINB) walk_mixed_kernel(const W
                         // branch-free four-step body schedules better
                     }
                     };
-                    if (kBlockInside && all_inside)
+                    if (kBlockTest && all_inside)
                         full_steps(std::true_type{});
                     else
                         full_steps(std::false_type{});
                 }
                 ++blk;
                 if (!alive) {  // every copy has its exit record: mark the item complete
-                    P.pp_steps[sh_item[t]] = sh_steps[t] | kDoneFlag;
+                    P.pp_steps[sh_item[t]] = (long long)(sh_steps[t] | (unsigned long long)kDoneFlag);
                     busy = false;
                 } else if (4 * (int64_t)blk >= P.max_steps) {
                     const unsigned long long it = sh_item[t];
                     atomicOr(SEG ? P.seg[sh_seg[t]].status : P.status, 1 << MCG_ERR_STEP_CAP);
                     // (no completion flag: the exit kernel writes NaN)
-                    P.pp_steps[it] = sh_steps[t] + (long long)__popc(alive) * 4 * (long long)blk;
+                    P.pp_steps[it] = (long long)sh_steps[t] + (long long)__popc(alive) * 4 * (long long)blk;
                     busy = false;
                 }
             }
             // enough lanes want new work: leave the block loop to refill them
-            if (__popc(__ballot_sync(kFull, !busy && !exhausted)) >= P.refill_min) break;
+            if (!drained && __popc(__ballot_sync(kFull, !busy)) >= P.refill_min) break;
         }
-        // warp-uniform flush of the partial sums (at most 16 blocks = 64 steps each)
-        sh_D[0][t] += (double)S0;
-        S0 = 0.f;
-        if (CRN) {
-            sh_D[1][t] += (double)S1;
-            sh_D[2][t] += (double)S2;
-            S1 = S2 = 0.f;
-        }
+        // warp-uniform flush of the partial sums: every 64 steps at most for
+        // single-precision sums, now and then for the exact counts
+        if (!kTwoValued<RHO> || (round & 63u) == 0u) flush();
     }
 }
 
@@ -1104,8 +1346,9 @@ int walk_blocks_per_sm(int precision, int rho_kind, int block, bool seg)
     return nb > 0 ? nb : 1;
 }
 
-cudaError_t launch_walk(const WalkParams& P, int precision, int block, cudaStream_t st)
+cudaError_t launch_walk(const WalkParams& P0, int precision, int block, cudaStream_t st)
 {
+    WalkParams P = P0;
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -1115,7 +1358,27 @@ cudaError_t launch_walk(const WalkParams& P, int precision, int block, cudaStrea
     const int per_sm = walk_blocks_per_sm(precision, kind, block, P.seg != nullptr);
     long long grid = (long long)sms * per_sm;
     const long long need = (long long)((P.total + (unsigned long long)block - 1ull) / (unsigned long long)block);
-    if (grid > need) grid = need > 0 ? need : 1;
+    P.quota = 32;
+    if (precision == MCG_MIXED) {
+        // Walks per warp.  With a warpful for every resident warp the lanes
+        // run a walk each; with fewer the walks are spread over all warps,
+        // up to kStripMax each, which run them as strips.  Where the line
+        // lies (prism, 20 walks per resident warp: strips 65 ms, full lanes
+        // in fewer warps 79 ms; 30 per warp: 84 against 94 ms):
+        const long long per_block = block / 32;
+        const long long per_warp = (long long)(P.total / (unsigned long long)(grid * per_block));
+        if (per_warp < 32) {
+            P.quota = (int32_t)(per_warp < 1 ? 1 : per_warp > (long long)kStripMax ? kStripMax : per_warp);
+            const long long spread = (long long)((P.total + (unsigned long long)per_block - 1ull) /
+                                                 (unsigned long long)per_block);
+            if (grid > spread) grid = spread;
+        } else if (grid > need) {
+            grid = need;
+        }
+    } else if (grid > need) {
+        grid = need > 0 ? need : 1;
+    }
+    if (grid < 1) grid = 1;
     const bool crn = P.crn != 0;
     if (precision == MCG_FP64) {
         if (P.seg) {
