@@ -766,15 +766,16 @@ __global__ void __launch_bounds__(128, MCG_MIXED_MINB) walk_mixed_kernel(const W
                 N0 = N1 = N2 = 0u;
                 __syncwarp();
             };
+            const uint32_t flushed_at = gblk;  // (the last regrouping)
             // the block at whose end a live walk has reached the step cap
             const int64_t cap_blk = (P.max_steps + 3) / 4;
             bool ended = false;  // the group's walk is complete or capped
             for (int r = 0; r < 16; ++r) {
                 // blocks of this round: up to k, not past the cap, and for a
                 // density that is summed in single precision not past the
-                // next flush (every 16 blocks)
+                // next flush (16 blocks after the last)
                 int kk = k;
-                if constexpr (kVoxel<RHO>) kk = min(kk, 16 - (int)(gblk & 15u));
+                if constexpr (kVoxel<RHO>) kk = min(kk, 16 - (int)((gblk - flushed_at) & 15u));
                 if ((int64_t)gblk + kk > cap_blk) kk = (int)(cap_blk - (int64_t)gblk);
                 const bool act = mine && l < kk;
                 float nr[6], cs[12];
@@ -971,7 +972,7 @@ __global__ void __launch_bounds__(128, MCG_MIXED_MINB) walk_mixed_kernel(const W
                 }
                 gblk += (uint32_t)kk;
                 if constexpr (kVoxel<RHO>) {
-                    if ((gblk & 15u) == 0u && l < NC && mine) {  // flush (k >= 2: two lanes may take three copies)
+                    if (((gblk - flushed_at) & 15u) == 0u && l < NC && mine) {  // flush (k >= 2: two lanes may take three copies)
                         for (int c = l; c < NC; c += k) {
                             sh_acc[c][slot] = flushed<RHO>(sh_acc[c][slot], value_of(sh_part[c][slot]));
                             sh_part[c][slot] = (Part)0;
@@ -1015,8 +1016,9 @@ __global__ void __launch_bounds__(128, MCG_MIXED_MINB) walk_mixed_kernel(const W
                 if (ne) busy = false;
             }
             __syncwarp();
-            if constexpr (kTwoValued<RHO>)
-                if ((round & 63u) == 0u) flush();  // counts stay below 2^22 (at most 2048 steps a round)
+            // single-precision sums whenever the warp regroups, as lanes do;
+            // counts now and then (at most 2048 steps a round: below 2^22)
+            if (!kTwoValued<RHO> || (round & 63u) == 0u) flush();
             continue;
         }
 
@@ -1158,8 +1160,9 @@ __global__ void __launch_bounds__(128, MCG_MIXED_MINB) walk_mixed_kernel(const W
                     busy = false;
                 }
             }
-            // enough lanes want new work: leave the block loop to refill them
-            if (!drained && __popc(__ballot_sync(kFull, !busy)) >= P.refill_min) break;
+            // enough walks have ended: leave the block loop to refill their
+            // lanes or to regroup
+            if (__popc(livem & ~__ballot_sync(kFull, busy)) >= P.refill_min) break;
         }
         // warp-uniform flush of the partial sums: every 64 steps at most for
         // single-precision sums, now and then for the exact counts
@@ -1364,10 +1367,13 @@ cudaError_t launch_walk(const WalkParams& P0, int precision, int block, cudaStre
         // run a walk each; with fewer the walks are spread over all warps,
         // up to kStripMax each, which run them as strips.  Where the line
         // lies (prism, 20 walks per resident warp: strips 65 ms, full lanes
-        // in fewer warps 79 ms; 30 per warp: 84 against 94 ms):
+        // in fewer warps 79 ms; 30 per warp: 84 against 94 ms).  A voxel
+        // grid always starts with full warps: the rounding of its single-
+        // precision sums follows the walks that share a warp, and 32
+        // consecutive items keep it the same however many SMs there are.
         const long long per_block = block / 32;
         const long long per_warp = (long long)(P.total / (unsigned long long)(grid * per_block));
-        if (per_warp < 32) {
+        if (per_warp < 32 && P.rho_kind != MCG_RHO_VOXEL) {
             P.quota = (int32_t)(per_warp < 1 ? 1 : per_warp > (long long)kStripMax ? kStripMax : per_warp);
             const long long spread = (long long)((P.total + (unsigned long long)per_block - 1ull) /
                                                  (unsigned long long)per_block);
