@@ -2,6 +2,7 @@
 // outside the walk: the Gaussian-random-field density grid and the boundary
 // tables of the Dirichlet data (the potential of the voxel model on the six
 // faces of the box, by prism summation).
+#include <algorithm>
 #include <cmath>
 
 #include <cuda_runtime.h>
@@ -51,9 +52,11 @@ __global__ void grf_smooth_kernel(const double* __restrict__ a, double* __restri
     b[v] = acc;
 }
 
-// Mean and population standard deviation of a (one block, fixed order:
-// strided Neumaier partial sums, then a pairwise tree).  out[0] = mean,
-// out[1] = std.
+// Mean and population standard deviation of a, in two passes of
+// `blocks` blocks: strided Neumaier partial sums per thread, a pairwise tree
+// per block into part[block]; whoever needs the total adds the blocks'
+// sums in order.  (One block alone took 4.5 ms for 128 x 128 x 64 voxels: an SM
+// does 1.6 double-precision additions a clock.)
 __device__ void neumaier_add(double& s, double& c, double x)
 {
     const double t = s + x;
@@ -62,46 +65,56 @@ __device__ void neumaier_add(double& s, double& c, double x)
     s = t;
 }
 
-__global__ void __launch_bounds__(1024) grf_moments_kernel(const double* __restrict__ a, int64_t n,
-                                                           double* __restrict__ out)
+constexpr int kMomentThreads = 256;
+
+__device__ double in_order(const double* part, int blocks)
 {
-    __shared__ double sh[1024];
-    const int t = threadIdx.x;
     double s = 0.0, c = 0.0;
-    for (int64_t i = t; i < n; i += 1024) neumaier_add(s, c, a[i]);
-    sh[t] = s + c;
-    __syncthreads();
-    for (int k = 512; k > 0; k >>= 1) {
-        if (t < k) sh[t] += sh[t + k];
-        __syncthreads();
-    }
-    const double mean = sh[0] / (double)n;
-    __syncthreads();
-    s = 0.0;
-    c = 0.0;
-    for (int64_t i = t; i < n; i += 1024) {
-        const double d = a[i] - mean;
-        neumaier_add(s, c, d * d);
-    }
-    sh[t] = s + c;
-    __syncthreads();
-    for (int k = 512; k > 0; k >>= 1) {
-        if (t < k) sh[t] += sh[t + k];
-        __syncthreads();
-    }
-    if (t == 0) {
-        out[0] = mean;
-        out[1] = sqrt(sh[0] / (double)n);
-    }
+    for (int b = 0; b < blocks; ++b) neumaier_add(s, c, part[b]);
+    return s + c;
 }
 
-__global__ void grf_transform_kernel(const double* __restrict__ a, int64_t n, const double* __restrict__ mom,
-                                     double amp, float* __restrict__ grid)
+// MEAN: sum of a.  Otherwise sum of (a - mean)^2, the mean from `means`.
+template <bool MEAN>
+__global__ void __launch_bounds__(kMomentThreads) grf_moments_kernel(const double* __restrict__ a, int64_t n,
+                                                                     const double* __restrict__ means,
+                                                                     double* __restrict__ part)
 {
-    const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (v >= n) return;
-    const double Z = (a[v] - mom[0]) / mom[1];
-    grid[v] = (float)(amp * (exp(Z) - 1.0));
+    __shared__ double sh[kMomentThreads];
+    const int t = threadIdx.x;
+    double mean = 0.0;
+    if (!MEAN) {
+        if (t == 0) sh[0] = in_order(means, gridDim.x) / (double)n;
+        __syncthreads();
+        mean = sh[0];
+        __syncthreads();
+    }
+    double s = 0.0, c = 0.0;
+    for (int64_t i = (int64_t)blockIdx.x * kMomentThreads + t; i < n; i += (int64_t)gridDim.x * kMomentThreads) {
+        const double d = MEAN ? a[i] : (a[i] - mean) * (a[i] - mean);
+        neumaier_add(s, c, d);
+    }
+    sh[t] = s + c;
+    __syncthreads();
+    for (int k = kMomentThreads / 2; k > 0; k >>= 1) {
+        if (t < k) sh[t] += sh[t + k];
+        __syncthreads();
+    }
+    if (t == 0) part[blockIdx.x] = sh[0];
+}
+
+__global__ void grf_transform_kernel(const double* __restrict__ a, int64_t n, const double* __restrict__ means,
+                                     const double* __restrict__ squares, int blocks, double amp,
+                                     float* __restrict__ grid)
+{
+    __shared__ double mom[2];
+    if (threadIdx.x == 0) mom[0] = in_order(means, blocks) / (double)n;
+    if (threadIdx.x == 32) mom[1] = sqrt(in_order(squares, blocks) / (double)n);
+    __syncthreads();
+    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
+        const double Z = (a[v] - mom[0]) / mom[1];
+        grid[v] = (float)(amp * (exp(Z) - 1.0));
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -299,8 +312,14 @@ int grf_density(uint64_t seed, int64_t nx, int64_t ny, int64_t nz, double sigma_
         a = b;
         b = t;
     }
-    grf_moments_kernel<<<1, 1024, 0, st>>>(a, n, mom);
-    grf_transform_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(a, n, mom, amp, grid_out);
+    // the blocks' sums go behind the filter's spare buffer's start, or, for a
+    // grid too small to lend one, into the 32 doubles behind both
+    const int blocks = (int)std::min<int64_t>(64, (n + 4095) / 4096);
+    double* part = blocks > 8 ? b : mom;
+    grf_moments_kernel<true><<<blocks, kMomentThreads, 0, st>>>(a, n, nullptr, part);
+    grf_moments_kernel<false><<<blocks, kMomentThreads, 0, st>>>(a, n, part, part + blocks);
+    const int64_t tb = std::min<int64_t>((n + 255) / 256, 1024);
+    grf_transform_kernel<<<(unsigned)tb, 256, 0, st>>>(a, n, part, part + blocks, blocks, amp, grid_out);
     const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? MCG_OK : set_error(MCG_ERR_CUDA, "grf kernels: %s", cudaGetErrorString(e));
 }
