@@ -6,24 +6,30 @@
 //  * sphere: -G M / r outside, -G M (3 a^2 - r^2) / (2 a^3) inside;
 //  * prism : Nagy's corner function F summed over the eight corners,
 //            Phi = -G rho [[[F]]], dPhi/dz = G rho [[[dF/dz]]];
-//  * voxel : the direct sum of the voxels' prism potentials regrouped by grid
-//            node: every node is a corner of up to eight cells, each adding
-//            its density with the corner's sign, so
+//  * voxel : the sum of the voxels' prism fields.  Cells near the point are
+//            summed by grid node: every node is a corner of up to eight cells,
+//            each adding its density with the corner's sign, so
 //              Phi(x) = -G sum_nodes w_n F(n - x),  w_n = sum_cells s rho,
 //            one corner-function evaluation per node instead of eight per
-//            cell (the node-summation form of the prism sum).  Double
-//            precision throughout, with compensated sums in a fixed order.
+//            cell, in double precision.  All other cells use the series of
+//            mcg_cell.cuh, its leading term in pairs of single-precision
+//            numbers.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
+#include "mcg_cell.cuh"
 #include "mcg_device.cuh"
 #include "mcg_internal.h"
 
 namespace mcg {
 
 namespace {
+
+constexpr int kFieldTerms = 3 + 6 + 10 + 15;
 
 struct FieldParams {
     int32_t kind;
@@ -33,6 +39,8 @@ struct FieldParams {
     const float* grid;        // voxel grid, x fastest
     int32_t nx, ny, nz;
     double org[3], sp[3];
+    double series[kFieldTerms];  // cell_series of a cell, up to P_8
+    double near;              // cells with a centre within this of the point (per axis) are summed by node
     const double* x;          // points, n x 3
     int64_t n;
     double* phi;
@@ -111,54 +119,179 @@ __global__ void field_closed_kernel(const FieldParams P)
     if (P.gz) P.gz[i] = gz;
 }
 
-__device__ __forceinline__ double cell(const FieldParams& P, int i, int j, int k)
-{
-    if (i < 0 || j < 0 || k < 0 || i >= P.nx || j >= P.ny || k >= P.nz) return 0.0;
-    return (double)__ldg(P.grid + i + (int64_t)P.nx * (j + (int64_t)P.ny * k));
-}
-
-// Voxel model by node summation: one block per point, threads stride over
-// the (nx+1)(ny+1)(nz+1) nodes with compensated partial sums, then one thread
-// adds the partials in thread order (deterministic).
+// ---------------------------------------------------------------------------
+// Voxel model.  A cluster of blocks per point (one block where there are
+// many points).  What bounds it: GB300 does 1.6 double-precision operations a
+// clock and SM against 128 single-precision ones, and a corner function takes
+// about 390 of them, so the sum over every node of a 128 x 128 x 64 grid
+// spent 0.9 ms a point and SM-wave in the double-precision pipe (231 ms for
+// 256 points).  Only the cells within kNearCells sides of the point need it;
+// the others take ~95 single-precision instructions: a thread runs a row of
+// cells (its Y, Z polynomials in registers), 16 columns of 256 rows at a time
+// through shared memory so that the grid is read in whole sectors.  Now
+// 2.5 ms (one point 0.29 ms; flat 16 x 128 x 64 cells 9.6 ms).  Error
+// against the 64-bit sum over all nodes: 0.6-2.8e-13 of the field as before,
+// which is that sum's own cancellation.
+// ---------------------------------------------------------------------------
 constexpr int kFieldThreads = 256;
+constexpr int kFieldCols = 16;
+constexpr double kNearCells = 6.0;
 
-__global__ void __launch_bounds__(kFieldThreads) field_voxel_kernel(const FieldParams P)
+template <bool CUBE>
+__global__ void __launch_bounds__(kFieldThreads, 2) field_voxel_kernel(const FieldParams P)
 {
-    __shared__ double sh[2][kFieldThreads];
-    const int64_t i = blockIdx.x;
-    const double x0 = P.x[3 * i], x1 = P.x[3 * i + 1], x2 = P.x[3 * i + 2];
-    const int64_t Nx = P.nx + 1, Ny = P.ny + 1, Nn = Nx * Ny * (int64_t)(P.nz + 1);
-    double sf = 0.0, cf = 0.0, sd = 0.0, cd = 0.0;
-    for (int64_t q = threadIdx.x; q < Nn; q += kFieldThreads) {
-        const int a = (int)(q % Nx), b = (int)((q / Nx) % Ny), c = (int)(q / (Nx * Ny));
-        // node (a, b, c) is the upper corner (sign +) of cell a-1 and the
-        // lower corner (sign -) of cell a along each axis
-        double w = 0.0;
+    namespace cg = cooperative_groups;
+    const cg::cluster_group cluster = cg::this_cluster();
+    const int parts = (int)cluster.num_blocks(), part = (int)cluster.block_rank();
+    __shared__ float tile[kFieldThreads][kFieldCols + 1];
+    __shared__ Pair sx[kFieldCols];     // X of the tile's columns
+    __shared__ float sp[kFieldTerms];   // the series for lengths in units of L
+    __shared__ double red[2][kFieldThreads / 32], total[2];
+    const int64_t i = blockIdx.x / parts;
+    const int t = threadIdx.x;
+    const double x[3] = {P.x[3 * i], P.x[3 * i + 1], P.x[3 * i + 2]};
+    const int n[3] = {P.nx, P.ny, P.nz};
+    // the near cells, and the unit of length: the geometric mean of the
+    // nearest and the farthest distance keeps r^8 and r^-17 within range
+    int lo[3], hi[3];  // near cells lo .. hi - 1 along each axis
+    double out2 = 0.0, far2 = 0.0;
+    for (int k = 0; k < 3; ++k) {
+        const double a = (x[k] - P.org[k]) / P.sp[k], w = P.near / P.sp[k];
+        lo[k] = (int)fmin(fmax(ceil(a - w - 0.5), 0.0), (double)n[k]);
+        hi[k] = (int)fmin(fmax(floor(a + w - 0.5) + 1.0, 0.0), (double)n[k]);
+        const double g0 = P.org[k] - x[k], g1 = g0 + n[k] * P.sp[k];
+        const double o = fmax(fmax(g0, -g1), 0.0), f = fmax(fabs(g0), fabs(g1));
+        out2 += o * o;
+        far2 += f * f;
+    }
+    const bool none_near = lo[0] >= hi[0] || lo[1] >= hi[1] || lo[2] >= hi[2];
+    if (none_near)
+        for (int k = 0; k < 3; ++k) lo[k] = hi[k] = 0;
+    const double L = sqrt(fmax(sqrt(out2), P.near) * sqrt(far2)), invL = 1.0 / L;
+    if (t < kFieldTerms) {
+        const double q = invL * invL;
+        sp[t] = (float)(P.series[t] * (t < 3 ? q : t < 9 ? q * q : t < 19 ? q * q * q : (q * q) * (q * q)));
+    }
+
+    // far cells: sum of rho f and of rho (df/dz), lengths in units of L
+    double phi = 0.0, gz = 0.0;
+    const int64_t rows = (int64_t)P.ny * P.nz;
+    const Pair p2x = pair_of(P.series[0] * invL * invL), p2z2 = pair_of(2.0 * P.series[2] * invL * invL);
+    for (int64_t r0 = (int64_t)part * kFieldThreads; r0 < rows; r0 += (int64_t)parts * kFieldThreads) {
+        const int64_t row = r0 + t;
+        const int iy = (int)(row % P.ny), iz = (int)(row / P.ny);
+        const double dy = (P.org[1] + (iy + 0.5) * P.sp[1] - x[1]) * invL,
+                     dz = (P.org[2] + (iz + 0.5) * P.sp[2] - x[2]) * invL;
+        const Pair yz = pair_of(dy * dy + dz * dz);
+        const Pair c2 = pair_of((P.series[1] * dy * dy + P.series[2] * dz * dz) * invL * invL);
+        SeriesRow sr;
+        Pair fs = {0.f, 0.f}, gs = {0.f, 0.f};  // the row's sums
+        for (int c0 = 0; c0 < P.nx; c0 += kFieldCols) {
+            __syncthreads();
+            for (int e = t; e < kFieldThreads * kFieldCols; e += kFieldThreads) {
+                const int er = e / kFieldCols, ec = e % kFieldCols;
+                const int64_t rr = r0 + er;
+                const int ix = c0 + ec;
+                float v = 0.f;
+                if (rr < rows && ix < P.nx) {
+                    const int jy = (int)(rr % P.ny), jz = (int)(rr / P.ny);
+                    const bool near = ix >= lo[0] && ix < hi[0] && jy >= lo[1] && jy < hi[1] && jz >= lo[2] && jz < hi[2];
+                    if (!near) v = __ldg(P.grid + rr * P.nx + ix);
+                }
+                tile[er][ec] = v;
+            }
+            if (t < kFieldCols) {
+                const double dx = (P.org[0] + (c0 + t + 0.5) * P.sp[0] - x[0]) * invL, X = dx * dx;
+                sx[t] = pair_of(X);
+            }
+            __syncthreads();
+            if (c0 == 0) sr = series_row(sp, (float)(dy * dy), (float)(dz * dz));
+            const int cols = P.nx - c0 < kFieldCols ? P.nx - c0 : kFieldCols;
+#pragma unroll 2
+            for (int c = 0; c < cols; ++c) {
+                const float rho = tile[t][c];
+                if (rho == 0.0f) continue;  // (near, outside the grid, or empty)
+                const Pair X = sx[c];
+                Pair y2;
+                const Pair y = rsqrt_pair(add(X, yz), y2);
+                float P4, P6, P8;
+                series_polys(sp, sr, X.h, P4, P6, P8);
+                Pair f = {y.h, y.l + series_value(P4, P6, P8, y.h, y2.h)};
+                const Pair y3 = mul(y, y2);
+                Pair g = {-y3.h, series_slope(sp, sr, X.h, P4, P6, P8, y.h, y2.h) - y3.l};
+                if constexpr (!CUBE) {
+                    Pair P2, y5;
+                    const Pair v = series_second(p2x, c2, X, y, y2, P2, y5);
+                    f = add_small(f, v);
+                    // 2 dP_2/dZ y^5 - 5 P_2 y^7
+                    const Pair w = mul(mul(P2, y2), {-5.0f, 0.0f});
+                    g = add_small(g, mul(add(p2z2, w), y5));
+                }
+                accumulate(fs, mul({rho, 0.0f}, f));
+                accumulate(gs, mul({rho, 0.0f}, g));
+            }
+        }
+        phi += (double)fs.h + (double)fs.l;
+        gz += dz * ((double)gs.h + (double)gs.l);
+    }
+    const double V = P.sp[0] * P.sp[1] * P.sp[2];
+    phi *= V * invL;
+    gz *= V * invL * invL;
+
+    // near cells: their nodes lo .. hi, each with the weight of the near
+    // cells it belongs to (upper corner, sign +, of the cell before it along
+    // an axis, lower corner, sign -, of its own)
+    if (!none_near) {
+        const int mx = hi[0] - lo[0] + 1, my = hi[1] - lo[1] + 1, mz = hi[2] - lo[2] + 1;
+        const int64_t nodes = (int64_t)mx * my * mz;
+        double sf = 0.0, cf = 0.0, sd = 0.0, cd = 0.0;
+        for (int64_t q = (int64_t)part * kFieldThreads + t; q < nodes; q += (int64_t)parts * kFieldThreads) {
+            const int a = lo[0] + (int)(q % mx), b = lo[1] + (int)((q / mx) % my), c = lo[2] + (int)(q / ((int64_t)mx * my));
+            double w = 0.0;
 #pragma unroll
-        for (int m = 0; m < 8; ++m) {
-            const int di = m & 1, dj = (m >> 1) & 1, dk = (m >> 2) & 1;
-            const double v = cell(P, a - 1 + di, b - 1 + dj, c - 1 + dk);
-            w += ((di + dj + dk) & 1) ? -v : v;
+            for (int m = 0; m < 8; ++m) {
+                const int di = m & 1, dj = (m >> 1) & 1, dk = (m >> 2) & 1;
+                const int ci = a - 1 + di, cj = b - 1 + dj, ck = c - 1 + dk;
+                double v = 0.0;
+                if (ci >= lo[0] && ci < hi[0] && cj >= lo[1] && cj < hi[1] && ck >= lo[2] && ck < hi[2])
+                    v = (double)__ldg(P.grid + ci + (int64_t)P.nx * (cj + (int64_t)P.ny * ck));
+                w += ((di + dj + dk) & 1) ? -v : v;
+            }
+            if (w == 0.0) continue;
+            double F, D;
+            corner_f_dfdz(P.org[0] + a * P.sp[0] - x[0], P.org[1] + b * P.sp[1] - x[1], P.org[2] + c * P.sp[2] - x[2],
+                          F, D);
+            neumaier(sf, cf, w * F);
+            neumaier(sd, cd, w * D);
         }
-        if (w == 0.0) continue;
-        double F, D;
-        corner_f_dfdz(P.org[0] + a * P.sp[0] - x0, P.org[1] + b * P.sp[1] - x1, P.org[2] + c * P.sp[2] - x2, F,
-                      D);
-        neumaier(sf, cf, w * F);
-        neumaier(sd, cd, w * D);
+        phi += sf + cf;
+        gz += sd + cd;
     }
-    sh[0][threadIdx.x] = sf + cf;
-    sh[1][threadIdx.x] = sd + cd;
+
+    // block sums, then the cluster's, in a fixed order
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        phi += __shfl_xor_sync(0xffffffffu, phi, o);
+        gz += __shfl_xor_sync(0xffffffffu, gz, o);
+    }
+    if ((t & 31) == 0) {
+        red[0][t >> 5] = phi;
+        red[1][t >> 5] = gz;
+    }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double s0 = 0.0, c0 = 0.0, s1 = 0.0, c1 = 0.0;
-        for (int t = 0; t < kFieldThreads; ++t) {
-            neumaier(s0, c0, sh[0][t]);
-            neumaier(s1, c1, sh[1][t]);
-        }
-        if (P.phi) P.phi[i] = -P.G * (s0 + c0);
-        if (P.gz) P.gz[i] = P.G * (s1 + c1);
+    if (t < 2) {
+        double v = 0.0;
+        for (int w = 0; w < kFieldThreads / 32; ++w) v += red[t][w];
+        total[t] = v;
     }
+    cluster.sync();
+    if (part == 0 && t < 2) {
+        double v = 0.0;
+        for (int b = 0; b < parts; ++b) v += *cluster.map_shared_rank(&total[t], b);
+        if (t == 0 && P.phi) P.phi[i] = -P.G * v;
+        if (t == 1 && P.gz) P.gz[i] = P.G * v;
+    }
+    cluster.sync();  // the other blocks' shared memory stays until it has been read
 }
 
 // The walks' own density samplers at given points and their two copies
@@ -192,13 +325,78 @@ __global__ void density_f64_kernel(const WalkParams P, const double* __restrict_
     }
 }
 
+// The integer polynomials d^(2i,2j,2k) (1 / r) r^(4n+1), n = i + j + k: one
+// derivative at a time, d_x (P / r^m) = (r^2 d_x P - m x P) / r^(m+2).
+struct DerivativeTable {
+    // [n-1][index of (i, j, k)][index of the monomial], both by falling first
+    // and second exponent
+    double c[kSeriesOrders][21][21];
+    DerivativeTable()
+    {
+        constexpr int N = 2 * kSeriesOrders + 1;  // exponents 0 .. 10
+        auto at = [](int a, int b, int c) { return (a * N + b) * N + c; };
+        std::memset(c, 0, sizeof(c));
+        for (int n = 1; n <= kSeriesOrders; ++n)
+            for (int i = n, e = 0; i >= 0; --i)
+                for (int j = n - i; j >= 0; --j, ++e) {
+                    const int order[3] = {2 * i, 2 * j, 2 * (n - i - j)};
+                    double P[N * N * N] = {};
+                    P[0] = 1.0;
+                    int m = 1, deg = 0;
+                    for (int ax = 0; ax < 3; ++ax)
+                        for (int d = 0; d < order[ax]; ++d, m += 2, ++deg) {
+                            double Q[N * N * N] = {};
+                            for (int a = 0; a <= deg; ++a)
+                                for (int b = 0; a + b <= deg; ++b) {
+                                    const int x[3] = {a, b, deg - a - b};
+                                    const double v = P[at(x[0], x[1], x[2])];
+                                    if (v == 0.0) continue;
+                                    int y[3] = {x[0], x[1], x[2]};
+                                    ++y[ax];
+                                    Q[at(y[0], y[1], y[2])] -= m * v;
+                                    if (x[ax] == 0) continue;
+                                    for (int k = 0; k < 3; ++k) {
+                                        int z[3] = {x[0], x[1], x[2]};
+                                        --z[ax];
+                                        z[k] += 2;
+                                        Q[at(z[0], z[1], z[2])] += x[ax] * v;
+                                    }
+                                }
+                            std::memcpy(P, Q, sizeof(P));
+                        }
+                    for (int a = n, q = 0; a >= 0; --a)
+                        for (int b = n - a; b >= 0; --b, ++q) c[n - 1][e][q] = P[at(2 * a, 2 * b, 2 * (n - a - b))];
+                }
+    }
+};
+
 }  // namespace
+
+void cell_series(const double h[3], double out[kSeriesTerms])
+{
+    static const DerivativeTable T;
+    const double fact[kSeriesOrders + 1] = {1.0, 6.0, 120.0, 5040.0, 362880.0, 39916800.0};  // (2i + 1)!
+    double* o = out;
+    for (int n = 1; n <= kSeriesOrders; ++n) {
+        const int terms = (n + 1) * (n + 2) / 2;
+        for (int q = 0; q < terms; ++q) o[q] = 0.0;
+        for (int i = n, e = 0; i >= 0; --i)
+            for (int j = n - i; j >= 0; --j, ++e) {
+                const int k = n - i - j;
+                const double w = std::pow(h[0], 2 * i) * std::pow(h[1], 2 * j) * std::pow(h[2], 2 * k) /
+                                 (fact[i] * fact[j] * fact[k]);
+                for (int q = 0; q < terms; ++q) o[q] += w * T.c[n - 1][e][q];
+            }
+        o += terms;
+    }
+}
 
 void preload_field_kernels()
 {
     cudaFuncAttributes a;
     if (cudaFuncGetAttributes(&a, (const void*)field_closed_kernel) != cudaSuccess) cudaGetLastError();
-    if (cudaFuncGetAttributes(&a, (const void*)field_voxel_kernel) != cudaSuccess) cudaGetLastError();
+    if (cudaFuncGetAttributes(&a, (const void*)field_voxel_kernel<true>) != cudaSuccess) cudaGetLastError();
+    if (cudaFuncGetAttributes(&a, (const void*)field_voxel_kernel<false>) != cudaSuccess) cudaGetLastError();
     const void* fns[6] = {(const void*)density_f64_kernel,           (const void*)density_f32_kernel<MCG_RHO_NONE>,
                           (const void*)density_f32_kernel<MCG_RHO_SPHERE>, (const void*)density_f32_kernel<MCG_RHO_PRISM>,
                           (const void*)density_f32_kernel<MCG_RHO_VOXEL>,  (const void*)density_f32_kernel<kRhoVoxelPacked>};
@@ -261,7 +459,27 @@ extern "C" int mcg_field(const mcg_density* density, const double* points_dev, i
             P.org[k] = density->origin[k];
             P.sp[k] = density->spacing[k];
         }
-        field_voxel_kernel<<<(unsigned)n, kFieldThreads, 0, st>>>(P);
+        const double half[3] = {0.5 * P.sp[0], 0.5 * P.sp[1], 0.5 * P.sp[2]};
+        double series[kSeriesTerms];
+        cell_series(half, series);
+        std::memcpy(P.series, series, sizeof(P.series));
+        P.near = kNearCells * std::max(P.sp[0], std::max(P.sp[1], P.sp[2]));
+        // few points: a cluster of eight blocks each, so that they fill the SMs
+        const unsigned parts = n < 2048 ? 8u : 1u;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)n * parts);
+        cfg.blockDim = dim3(kFieldThreads);
+        cfg.stream = st;
+        cudaLaunchAttribute at;
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = parts;
+        at.val.clusterDim.y = at.val.clusterDim.z = 1;
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        const bool cube = P.series[0] == 0.0 && P.series[1] == 0.0 && P.series[2] == 0.0;
+        const cudaError_t le = cube ? cudaLaunchKernelEx(&cfg, field_voxel_kernel<true>, P)
+                                    : cudaLaunchKernelEx(&cfg, field_voxel_kernel<false>, P);
+        if (le != cudaSuccess) return set_error(MCG_ERR_CUDA, "field kernel launch: %s", cudaGetErrorString(le));
         break;
     }
     default:
