@@ -5,8 +5,10 @@
 #include <algorithm>
 #include <cmath>
 
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
+#include "mcg_cell.cuh"
 #include "mcg_device.cuh"
 #include "mcg_internal.h"
 
@@ -128,12 +130,24 @@ struct TableParams {
     double org[3], sp[3];
     double vol;              // cell volume
     double near2;            // squared radius of the exact (near) zone
+    double unit;             // longest side of a cell
+    double second[3];        // cell_series for lengths in units of `unit`: its order 2 ...
+    float series[kSeriesTerms];  // ... and all of it in single precision
     double G;
     float* out;
 };
 
 constexpr int kTableThreads = 256;
+constexpr int kTableWarps = kTableThreads / 32;
 constexpr int kRowsPerTile = 8;
+// In units of the longest side, along every axis: cells up to kCoreSides from
+// the node are summed by grid node (exact); of the others in the near zone
+// those up to kExactSides as exact prisms (there are some only where the zone
+// is smaller than the core), the rest by the series of mcg_cell.cuh, whose
+// remainder beyond the core is about 1e-11 of the cell's own term: with the
+// core at three sides and without P_10 (1e-8) one table value in a thousand
+// rounded to its neighbour.
+constexpr double kCoreSides = 4.0, kExactSides = 2.0;
 
 __device__ __forceinline__ void node_position(const TableParams& T, int64_t node, double x[3])
 {
@@ -149,76 +163,192 @@ __device__ __forceinline__ void node_position(const TableParams& T, int64_t node
 }
 
 // Point-mass far field for every voxel (single-precision terms, summed per
-// row in single precision and per row into double), then the exact prism
-// potential in place of the point mass for voxels whose centre lies within
-// the near radius.  Writes Phi = -G sum.
-__global__ void __launch_bounds__(kTableThreads) tables_kernel(const TableParams T)
+// row in single precision and per row into double), then, for voxels whose
+// centre lies within the near radius, their own potential in place of the
+// point mass.  Writes Phi = -G sum.
+//
+// A block takes 32 NPL nodes (NPL per lane); its warps, and with few nodes the
+// blocks of its cluster, split the rows of the grid between them.  What
+// bounds it: the reciprocal root of each voxel and node (16 a clock and SM,
+// 22 ms for 6 x 128^2 nodes over 128 x 128 x 64 voxels).  Before, a thread
+// summed a node alone (486 nodes: 179 ms, on two SMs) and the near zone was
+// exact prisms in double precision throughout (6 x 128^2 nodes: 342 of 377 ms,
+// ~690 prisms a node of 8 corners; the pipe does 1.6 operations a clock and
+// SM).  Now 0.5 and 37 ms, 25 of them the point masses, with the same values
+// to the last bit.
+template <int NPL>
+__global__ void __launch_bounds__(kTableThreads, 2) tables_kernel(const TableParams T)
 {
-    __shared__ float rho_s[kRowsPerTile][128];
-    __shared__ float cx_s[128];  // voxel-centre x offsets, (float)ix * sx
+    namespace cg = cooperative_groups;
+    const cg::cluster_group cluster = cg::this_cluster();
+    const int parts = (int)cluster.num_blocks(), part = (int)cluster.block_rank();
+    __shared__ float4 rho_s[kTableWarps][kRowsPerTile][32];
+    __shared__ float4 cx_s[32];                     // voxel-centre x offsets, (float)ix * sx
+    __shared__ double sum_s[kTableWarps][32 * NPL];
+    __shared__ double total_s[32 * NPL];
     const int64_t nodes = 6ll * T.nu * T.nv;
-    const int64_t node = (int64_t)blockIdx.x * kTableThreads + threadIdx.x;
-    double x[3] = {0.0, 0.0, 0.0};
-    if (node < nodes) node_position(T, node, x);
-    // node relative to the first voxel centre, single precision
-    const float px = (float)(x[0] - (T.org[0] + 0.5 * T.sp[0]));
-    const float py = (float)(x[1] - (T.org[1] + 0.5 * T.sp[1]));
-    const float pz = (float)(x[2] - (T.org[2] + 0.5 * T.sp[2]));
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t first = (int64_t)(blockIdx.x / parts) * (32 * NPL);
     const float sx = (float)T.sp[0], sy = (float)T.sp[1], sz = (float)T.sp[2];
-    for (int i = threadIdx.x; i < 128; i += kTableThreads) cx_s[i] = (float)i * sx;
-    double acc = 0.0;
-    const int rows = T.ny * T.nz;
-    for (int r0 = 0; r0 < rows; r0 += kRowsPerTile) {
-        __syncthreads();
-        for (int i = threadIdx.x; i < kRowsPerTile * 128; i += kTableThreads) {
-            const int rr = i / 128, ix = i % 128;
-            const int row = r0 + rr;
-            rho_s[rr][ix] = (row < rows && ix < T.nx) ? __ldg(T.grid + (int64_t)row * T.nx + ix) : 0.0f;
-        }
-        __syncthreads();
+    // (a column past the grid has no density: far away, so that its term is 0)
+    for (int i = threadIdx.x; i < 128; i += kTableThreads) ((float*)cx_s)[i] = i < T.nx ? (float)i * sx : 1e18f;
+    __syncthreads();
+    float px[NPL], py[NPL], pz[NPL];
+    double acc[NPL];
+#pragma unroll
+    for (int j = 0; j < NPL; ++j) {
+        const int64_t node = first + 32 * j + lane;
+        double x[3];
+        node_position(T, node < nodes ? node : nodes - 1, x);
+        // node relative to the first voxel centre, single precision
+        px[j] = (float)(x[0] - (T.org[0] + 0.5 * T.sp[0]));
+        py[j] = (float)(x[1] - (T.org[1] + 0.5 * T.sp[1]));
+        pz[j] = (float)(x[2] - (T.org[2] + 0.5 * T.sp[2]));
+        acc[j] = 0.0;
+    }
+    const int rows = T.ny * T.nz, quads = (T.nx + 3) / 4;
+    const int stride = kTableWarps * parts * kRowsPerTile;
+    for (int r0 = (part * kTableWarps + warp) * kRowsPerTile; r0 < rows; r0 += stride) {
+        __syncwarp();
+        for (int rr = 0; rr < kRowsPerTile; ++rr)
+            for (int ix = lane; ix < 4 * quads; ix += 32)
+                ((float*)rho_s[warp][rr])[ix] =
+                    (r0 + rr < rows && ix < T.nx) ? __ldg(T.grid + (int64_t)(r0 + rr) * T.nx + ix) : 0.0f;
+        __syncwarp();
         for (int rr = 0; rr < kRowsPerTile && r0 + rr < rows; ++rr) {
             const int row = r0 + rr;
-            const float dy = (float)(row % T.ny) * sy - py;
-            const float dz = (float)(row / T.ny) * sz - pz;
-            const float dyz2 = fmaf(dy, dy, dz * dz);
-            float part = 0.0f;
-            for (int ix = 0; ix < T.nx; ++ix) {
-                const float dx = cx_s[ix] - px;
-                part = fmaf(rho_s[rr][ix], rsqrtf(fmaf(dx, dx, dyz2)), part);
+            float dyz2[NPL], sum[NPL];
+#pragma unroll
+            for (int j = 0; j < NPL; ++j) {
+                const float dy = (float)(row % T.ny) * sy - py[j];
+                const float dz = (float)(row / T.ny) * sz - pz[j];
+                dyz2[j] = fmaf(dy, dy, dz * dz);
+                sum[j] = 0.0f;
             }
-            acc += (double)part;
+#pragma unroll 2
+            for (int q = 0; q < quads; ++q) {
+                const float4 r4 = rho_s[warp][rr][q], c4 = cx_s[q];
+                const float rv[4] = {r4.x, r4.y, r4.z, r4.w}, cv[4] = {c4.x, c4.y, c4.z, c4.w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+#pragma unroll
+                    for (int j = 0; j < NPL; ++j) {
+                        const float dx = cv[e] - px[j];
+                        float y;
+                        asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(fmaf(dx, dx, dyz2[j])));
+                        sum[j] = fmaf(rv[e], y, sum[j]);
+                    }
+            }
+#pragma unroll
+            for (int j = 0; j < NPL; ++j) acc[j] += (double)sum[j];
         }
     }
-    if (node >= nodes) return;
-    acc *= T.vol;
-    // near zone: exact prism minus the point mass already counted
-    const double R = sqrt(T.near2);
-    int ilo[3], ihi[3];
+    // near zone: the voxel's own potential minus the point mass already
+    // counted; the rows of the zone's box go round the warps
+    const double R = sqrt(T.near2), inv = 1.0 / T.unit, inv2 = inv * inv;
     const int n[3] = {T.nx, T.ny, T.nz};
-    for (int k = 0; k < 3; ++k) {
-        const double a = fmin(fmax(floor((x[k] - R - T.org[k]) / T.sp[k]), 0.0), (double)n[k]);
-        const double b = fmin(fmax(floor((x[k] + R - T.org[k]) / T.sp[k]), -1.0), (double)(n[k] - 1));
-        ilo[k] = (int)a;
-        ihi[k] = (int)b;
-    }
-    for (int iz = ilo[2]; iz <= ihi[2]; ++iz)
-        for (int iy = ilo[1]; iy <= ihi[1]; ++iy)
+#pragma unroll
+    for (int j = 0; j < NPL; ++j) {
+        const int64_t node = first + 32 * j + lane;
+        double x[3];
+        node_position(T, node < nodes ? node : nodes - 1, x);
+        acc[j] *= T.vol;
+        int ilo[3], ihi[3];
+        for (int k = 0; k < 3; ++k) {
+            const double a = fmin(fmax(floor((x[k] - R - T.org[k]) / T.sp[k]), 0.0), (double)n[k]);
+            const double b = fmin(fmax(floor((x[k] + R - T.org[k]) / T.sp[k]), -1.0), (double)(n[k] - 1));
+            ilo[k] = (int)a;
+            ihi[k] = (int)b;
+        }
+        if (ilo[0] > ihi[0] || ilo[1] > ihi[1] || ilo[2] > ihi[2]) continue;
+        // the core: a box of cells inside the near zone
+        const double core = fmin(kCoreSides * T.unit, R * 0.57);
+        int clo[3], chi[3];
+        for (int k = 0; k < 3; ++k) {
+            const double a = (x[k] - T.org[k]) / T.sp[k], w = core / T.sp[k];
+            clo[k] = (int)fmin(fmax(ceil(a - w - 0.5), 0.0), (double)n[k]);
+            chi[k] = (int)fmin(fmax(floor(a + w - 0.5) + 1.0, 0.0), (double)n[k]);
+        }
+        const int wy = ihi[1] - ilo[1] + 1, box_rows = wy * (ihi[2] - ilo[2] + 1);
+        for (int q = part * kTableWarps + warp; q < box_rows; q += kTableWarps * parts) {
+            const int iy = ilo[1] + q % wy, iz = ilo[2] + q / wy;
+            const double cy = T.org[1] + (iy + 0.5) * T.sp[1] - x[1], cz = T.org[2] + (iz + 0.5) * T.sp[2] - x[2];
+            const double cyz = cy * cy + cz * cz;
+            if (cyz >= T.near2) continue;
+            const bool core_row = iy >= clo[1] && iy < chi[1] && iz >= clo[2] && iz < chi[2];
+            const bool exact_row = fabs(cy) < kExactSides * T.unit && fabs(cz) < kExactSides * T.unit;
+            const double Y = cy * cy * inv2, Z = cz * cz * inv2;
+            const SeriesRow sr = series_row(T.series, (float)Y, (float)Z);
+            const Pair p2x = pair_of(T.second[0]), c2 = pair_of(T.second[1] * Y + T.second[2] * Z);
+            const float dy = (float)iy * sy - py[j], dz = (float)iz * sz - pz[j];
             for (int ix = ilo[0]; ix <= ihi[0]; ++ix) {
                 const double cx = T.org[0] + (ix + 0.5) * T.sp[0] - x[0];
-                const double cy = T.org[1] + (iy + 0.5) * T.sp[1] - x[1];
-                const double cz = T.org[2] + (iz + 0.5) * T.sp[2] - x[2];
-                if (cx * cx + cy * cy + cz * cz >= T.near2) continue;
+                const double d2 = cx * cx + cyz;
+                if (d2 >= T.near2) continue;
                 const float rho = __ldg(T.grid + ((int64_t)iz * T.ny + iy) * T.nx + ix);
                 if (rho == 0.0f) continue;
-                const double lo[3] = {T.org[0] + ix * T.sp[0], T.org[1] + iy * T.sp[1], T.org[2] + iz * T.sp[2]};
-                const double hi[3] = {lo[0] + T.sp[0], lo[1] + T.sp[1], lo[2] + T.sp[2]};
-                // prism_potential returns -G rho [[[F]]]; with G = -1 it gives +rho [[[F]]]
-                const double exact = prism_potential(-1.0, (double)rho, lo, hi, x);
-                const float dx = cx_s[ix] - px, dy = (float)iy * sy - py, dz = (float)iz * sz - pz;
-                const double pm = T.vol * (double)(rho * rsqrtf(fmaf(dx, dx, fmaf(dy, dy, dz * dz))));
-                acc += exact - pm;
+                const float dx = ((const float*)cx_s)[ix] - px[j];
+                float pm;
+                asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(pm) : "f"(fmaf(dx, dx, fmaf(dy, dy, dz * dz))));
+                if (core_row && ix >= clo[0] && ix < chi[0]) {
+                    acc[j] -= T.vol * (double)(rho * pm);  // its own potential: the core's node sum
+                } else if (exact_row && fabs(cx) < kExactSides * T.unit) {
+                    const double lo[3] = {T.org[0] + ix * T.sp[0], T.org[1] + iy * T.sp[1], T.org[2] + iz * T.sp[2]};
+                    const double hi[3] = {lo[0] + T.sp[0], lo[1] + T.sp[1], lo[2] + T.sp[2]};
+                    // (returns -G rho [[[F]]]; with G = -1 it gives +rho [[[F]]])
+                    const double exact = prism_potential_paired(-1.0, (double)rho, lo, hi, x);
+                    acc[j] += exact - T.vol * (double)(rho * pm);
+                } else {
+                    const Pair X = pair_of(cx * cx * inv2);
+                    Pair y2, P2, y5;
+                    const Pair y = rsqrt_pair(pair_of(d2 * inv2), y2);
+                    const Pair v = series_second(p2x, c2, X, y, y2, P2, y5);
+                    float P4, P6, P8;
+                    series_polys(T.series, sr, X.h, P4, P6, P8);
+                    const Pair f = add_small(
+                        {y.h, y.l + (series_value(P4, P6, P8, y.h, y2.h) + series_tenth(T.series, sr, X.h, y.h, y2.h))}, v);
+                    acc[j] += T.vol * ((double)rho * (((double)f.h + (double)f.l) * inv) - (double)(rho * pm));
+                }
             }
-    T.out[node] = (float)(-T.G * acc);
+        }
+        // the core's nodes, each with the weight of the core cells it belongs
+        // to (upper corner, sign +, of the cell before it along an axis,
+        // lower corner, sign -, of its own)
+        const int mx = chi[0] - clo[0] + 1, my = chi[1] - clo[1] + 1, mz = chi[2] - clo[2] + 1;
+        if (mx <= 1 || my <= 1 || mz <= 1) continue;
+        for (int q = part * kTableWarps + warp; q < mx * my * mz; q += kTableWarps * parts) {
+            const int a = clo[0] + q % mx, b = clo[1] + q / mx % my, c = clo[2] + q / (mx * my);
+            double w = 0.0;
+#pragma unroll
+            for (int m = 0; m < 8; ++m) {
+                const int ci = a - 1 + (m & 1), cj = b - 1 + ((m >> 1) & 1), ck = c - 1 + (m >> 2);
+                double v = 0.0;
+                if (ci >= clo[0] && ci < chi[0] && cj >= clo[1] && cj < chi[1] && ck >= clo[2] && ck < chi[2])
+                    v = (double)__ldg(T.grid + ((int64_t)ck * T.ny + cj) * T.nx + ci);
+                w += ((m ^ (m >> 1) ^ (m >> 2)) & 1) ? -v : v;
+            }
+            if (w != 0.0)
+                acc[j] += w * prism_corner(T.org[0] + a * T.sp[0] - x[0], T.org[1] + b * T.sp[1] - x[1],
+                                           T.org[2] + c * T.sp[2] - x[2]);
+        }
+    }
+    // the warps' sums, then the cluster's, in order
+#pragma unroll
+    for (int j = 0; j < NPL; ++j) sum_s[warp][32 * j + lane] = acc[j];
+    __syncthreads();
+    const int t = threadIdx.x;
+    if (t < 32 * NPL) {
+        double v = 0.0;
+        for (int w = 0; w < kTableWarps; ++w) v += sum_s[w][t];
+        total_s[t] = v;
+    }
+    cluster.sync();
+    if (part == 0 && t < 32 * NPL && first + t < nodes) {
+        double v = 0.0;
+        for (int b = 0; b < parts; ++b) v += *cluster.map_shared_rank(&total_s[t], b);
+        T.out[first + t] = (float)(-T.G * v);
+    }
+    cluster.sync();  // the other blocks' shared memory stays until it has been read
 }
 
 // Packed voxel grid: entry (iz + 1, iy, ix) = layers iz-1, iz, iz+1 of
@@ -354,8 +484,32 @@ int boundary_tables(const mcg_domain* d, const mcg_density* rho, int32_t nu, int
     T.G = rho->G;
     T.out = faces_out;
     const int64_t nodes = 6ll * nu * nv;
-    tables_kernel<<<(unsigned)((nodes + kTableThreads - 1) / kTableThreads), kTableThreads, 0, st>>>(T);
-    const cudaError_t e = cudaGetLastError();
+    T.unit = std::max(T.sp[0], std::max(T.sp[1], T.sp[2]));
+    const double half[3] = {0.5 * T.sp[0] / T.unit, 0.5 * T.sp[1] / T.unit, 0.5 * T.sp[2] / T.unit};
+    double series[kSeriesTerms];
+    cell_series(half, series);
+    for (int i = 0; i < 3; ++i) T.second[i] = series[i];
+    for (int i = 0; i < kSeriesTerms; ++i) T.series[i] = (float)series[i];
+    // two nodes a lane share each density read; with few nodes one, and a
+    // cluster of eight blocks for each 32 of them, so that they fill the SMs
+    int dev = 0, sms = 152;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const bool many = nodes >= 64ll * 4 * sms;
+    const int64_t per = many ? 64 : 32, groups = (nodes + per - 1) / per;
+    const unsigned parts = groups >= 4ll * sms ? 1u : 8u;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)groups * parts);
+    cfg.blockDim = dim3(kTableThreads);
+    cfg.stream = st;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = parts;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    const cudaError_t e = many ? cudaLaunchKernelEx(&cfg, tables_kernel<2>, T)
+                               : cudaLaunchKernelEx(&cfg, tables_kernel<1>, T);
     return e == cudaSuccess ? MCG_OK : set_error(MCG_ERR_CUDA, "tables kernel: %s", cudaGetErrorString(e));
 }
 
