@@ -33,8 +33,9 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint32_t k0, uint32_t k1
 }
 
 // ---------------------------------------------------------------------------
-// Double precision normals (the plain FP64 walk): u = (w + 1/2) 2^-32,
-// r = sqrt(-2 ln u1), angle 2 pi u2, cosine first.
+// Double precision normals (the random density; the FP64 walk's are in
+// mcg_fixed.cuh): u = (w + 1/2) 2^-32, r = sqrt(-2 ln u1), angle 2 pi u2,
+// cosine first.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ double u01_f64(uint32_t w) { return ((double)w + 0.5) * 0x1p-32; }
 
@@ -46,17 +47,6 @@ __device__ __forceinline__ void box_muller_f64(uint32_t w1, uint32_t w2, double&
     sincos(a, &sn, &cs);
     z0 = r * cs;
     z1 = r * sn;
-}
-
-__device__ __forceinline__ void normals12_f64(uint32_t s, uint32_t p, uint32_t b, uint32_t k0, uint32_t k1,
-                                              double z[12])
-{
-#pragma unroll
-    for (uint32_t i = 0; i < 3; ++i) {
-        const uint4 w = philox4x32_10(make_uint4(3u * b + i, p, s, 0u), k0, k1);
-        box_muller_f64(w.x, w.y, z[4 * i], z[4 * i + 1]);
-        box_muller_f64(w.z, w.w, z[4 * i + 2], z[4 * i + 3]);
-    }
 }
 
 // ---------------------------------------------------------------------------

@@ -128,6 +128,11 @@ cudaError_t reset_walk(const WalkParams& P, cudaStream_t st);
 // Kernel launchers (mcg_walk.cu).
 cudaError_t launch_walk(const WalkParams& P, int precision, int block, cudaStream_t st);
 int walk_blocks_per_sm(int precision, int rho_kind, int block, bool seg = false);
+// The double-precision walk (mcg_walk64.cu): its kernel, and its launch on at
+// most `blocks` blocks.
+const void* walk64_fn(int rho_kind, bool crn, bool seg);
+cudaError_t launch_walk64(const WalkParams& P, int block, int blocks, cudaStream_t st);
+void preload_walk64_kernels();
 
 // Reduction launchers (mcg_reduce.cu).
 cudaError_t launch_reduce(const double* pp_u, const double* pp_d, const int64_t* pp_steps, int64_t S,

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include "mcg_device.cuh"
+#include "mcg_fixed.cuh"
 #include "mcg_internal.h"
 
 namespace mcg {
@@ -24,9 +25,17 @@ __global__ void normals_f64_kernel(uint32_t k0, uint32_t k1, uint32_t s, uint32_
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= nb) return;
-    double z[12];
-    normals12_f64(s, p, b0 + (uint32_t)i, k0, k1, z);
-    for (int j = 0; j < 12; ++j) out[12 * i + j] = z[j];
+    for (uint32_t j = 0; j < 3; ++j) {
+        const uint4 w = philox4x32_10(make_uint4(3u * (b0 + (uint32_t)i) + j, p, s, 0u), k0, k1);
+        for (int q = 0; q < 2; ++q) {
+            double r;
+            float rf;
+            int64_t co, si;
+            fx::polar64(fx::g_tables, q ? w.z : w.x, q ? w.w : w.y, r, rf, co, si);
+            out[12 * i + 4 * j + 2 * q] = __dmul_rn(r, __ll2double_rn(co));
+            out[12 * i + 4 * j + 2 * q + 1] = __dmul_rn(r, __ll2double_rn(si));
+        }
+    }
 }
 
 __global__ void normals_f32_kernel(uint32_t k0, uint32_t k1, uint32_t s, uint32_t p, uint32_t b0, int64_t nb,

@@ -1,6 +1,7 @@
-// mcg_walk.cu -- the walk kernels (Sec. 2.3 of the paper, steps 1-4).
+// mcg_walk.cu -- the mixed walk (Sec. 2.3 of the paper, steps 1-4) and the
+// launch of either walk (the double-precision one is in mcg_walk64.cu).
 //
-// Both kernels are persistent: every warp keeps 32 walks in flight and, as
+// The kernel is persistent: every warp keeps up to 32 walks in flight and, as
 // walks exit, refills the free lanes from a global work counter with one
 // warp-aggregated atomic (__ballot_sync / __shfl_sync), so lanes do not idle
 // behind the long exit-time tail.  A lane owns one path (station s, path p)
@@ -8,10 +9,6 @@
 // every Gaussian increment.  Random numbers come four steps at a time: three
 // Philox4x32-10 calls -> twelve normals -> four Euler-Maruyama steps.
 //
-//  * walk_fp64_kernel : the plain double-precision walk; its arithmetic
-//    follows the problem statement operation by operation (no contraction)
-//    so that a path agrees with a plain double-precision evaluation to
-//    rounding of the transcendental functions.
 //  * walk_mixed_kernel: single-precision stepping, random-number transform
 //    and density lookup; the source integral keeps single-precision partial
 //    sums over at most 64 steps which are flushed into a double accumulator
@@ -29,6 +26,7 @@
 
 #include "mcg_device.cuh"
 #include "mcg_internal.h"
+#include "mcg_walk.cuh"
 
 namespace mcg {
 
@@ -37,69 +35,6 @@ namespace {
 #ifndef MCG_MIXED_MINB
 #define MCG_MIXED_MINB 5
 #endif
-
-constexpr unsigned kFull = 0xffffffffu;
-constexpr double kNaN = __builtin_nan("");
-
-
-// Claims new items for free lanes of this warp while it holds fewer than
-// `quota` walks.  Returns true on the lanes that got one (in `item`); sets
-// the warp-uniform `drained` once the work list has no more.
-__device__ __forceinline__ bool refill(const WalkParams& P, bool busy, unsigned quota, bool& drained,
-                                       unsigned long long& item)
-{
-    const unsigned freem = __ballot_sync(kFull, !busy);
-    const unsigned live = 32u - (unsigned)__popc(freem);
-    if (drained || live >= quota) return false;
-    const int lane = threadIdx.x & 31;
-    const unsigned rank = (unsigned)__popc(freem & ((1u << lane) - 1u));
-    const bool want = !busy && rank < quota - live;
-    const unsigned wantm = __ballot_sync(kFull, want);
-    const int leader = __ffs(wantm) - 1;
-    unsigned long long base = 0ull;
-    if (lane == leader) base = atomicAdd(P.counter, (unsigned long long)__popc(wantm));
-    base = __shfl_sync(kFull, base, leader);
-    drained = base + (unsigned long long)__popc(wantm) >= P.total;
-    item = base + rank;  // the wanting lanes are the first of the free ones
-    return want && item < P.total;
-}
-
-// A station whose walk copies are not all strictly inside Omega gets NaN
-// and the MCG_ERR_ARG bit (mcgrav_solve rejects such stations up front).
-__device__ __forceinline__ bool station_ok(const WalkParams& P, const double* stations, int32_t* status, uint32_t s,
-                                           unsigned long long item)
-{
-    const double x = stations[3 * s], y = stations[3 * s + 1], z = stations[3 * s + 2];
-    bool ok;
-    if (P.ball) {
-        const double dx = x - P.cen[0], dy = y - P.cen[1], dz = z - P.cen[2];
-        const double q = dx * dx + dy * dy;
-        ok = q + dz * dz < P.R2 && q + (dz + P.h) * (dz + P.h) < P.R2 && q + (dz - P.h) * (dz - P.h) < P.R2;
-    } else {
-        ok = x > P.lo[0] && x < P.hi[0] && y > P.lo[1] && y < P.hi[1] && z - P.h > P.lo[2] && z + P.h < P.hi[2] &&
-             z > P.lo[2] && z < P.hi[2];
-    }
-    if (!ok) {
-        P.pp_u[item] = kNaN;
-        P.pp_d[item] = kNaN;
-        P.pp_steps[item] = 0;  // no completion flag: the mixed walk's exit kernel writes NaN too
-        atomicOr(status, 1 << MCG_ERR_ARG);
-    }
-    return ok;
-}
-
-__device__ __forceinline__ int64_t nstep_of(uint32_t blk, int m) { return 4 * (int64_t)blk + m + 1; }
-
-// The cancel flag may live in host-mapped or device memory and is written
-// by the host while the kernel runs: read it with a system-scope relaxed
-// load so the write is observed whatever caches the line.
-__device__ __forceinline__ bool cancelled(const WalkParams& P)
-{
-    int c = 0;
-    if ((threadIdx.x & 31) == 0 && P.cancel != nullptr)
-        asm volatile("ld.relaxed.sys.global.s32 %0, [%1];" : "=r"(c) : "l"((const void*)P.cancel) : "memory");
-    return __shfl_sync(kFull, c, 0) != 0;
-}
 
 // ---------------------------------------------------------------------------
 // Bounded wait on a hand-over slot (failure-detection hook).  Walks stay in
@@ -138,69 +73,6 @@ __device__ __forceinline__ void pool_wait(const WalkParams& P)
         if (!ready) __nanosleep(64);
     }
     if (!ready) atomicOr(P.status, 1 << MCG_ERR_TIMEOUT);
-}
-
-// Fraction theta in [0, 1] of the step X -> X + dW (coordinates relative to
-// the ball centre) at which the segment leaves the ball of radius R: the
-// positive root of |X + theta dW|^2 = R^2 in the form without cancellation.
-__device__ __forceinline__ double ball_theta(const double* q, const double* dW, double R2)
-{
-    double a = 0.0, b = 0.0, c = -R2;
-    for (int k = 0; k < 3; ++k) {
-        a = __dadd_rn(a, __dmul_rn(dW[k], dW[k]));
-        b = __dadd_rn(b, __dmul_rn(__dmul_rn(2.0, q[k]), dW[k]));
-        c = __dadd_rn(c, __dmul_rn(q[k], q[k]));
-    }
-    const double D = __dadd_rn(__dmul_rn(b, b), -__dmul_rn(__dmul_rn(4.0, a), c));
-    const double t = (b >= 0.0) ? __ddiv_rn(__dmul_rn(-2.0, c), __dadd_rn(b, __dsqrt_rn(D)))
-                                : __ddiv_rn(__dadd_rn(-b, __dsqrt_rn(D)), __dmul_rn(2.0, a));
-    return fmin(fmax(t, 0.0), 1.0);
-}
-
-// ---------------------------------------------------------------------------
-// Exit handling (double precision).  X: last inside point, Y: first point
-// not strictly inside, both as the walk computed them.  Clips the segment at
-// its first boundary crossing (lowest axis on ties), closes the trapezoid
-// over the clipped part and returns g(x*) - 2 pi G I.
-// ---------------------------------------------------------------------------
-__device__ __noinline__ double exit_fp64(const WalkParams& P, const ModelRef& M, const double* X, const double* dW,
-                                         const double* Y, double I, double rp)
-{
-    double xs[3];
-    double theta = 1.0;
-    int face = -1;
-    if (P.clip && P.ball) {
-        const double q[3] = {__dadd_rn(X[0], -P.cen[0]), __dadd_rn(X[1], -P.cen[1]), __dadd_rn(X[2], -P.cen[2])};
-        theta = ball_theta(q, dW, P.R2);
-        for (int k = 0; k < 3; ++k) xs[k] = __dadd_rn(X[k], __dmul_rn(theta, dW[k]));
-    } else if (P.clip) {
-        int kstar = -1;
-        double tmin = __longlong_as_double(0x7ff0000000000000LL), bstar = 0.0;
-        for (int k = 0; k < 3; ++k) {
-            double b;
-            if (Y[k] <= P.lo[k]) b = P.lo[k];
-            else if (Y[k] >= P.hi[k]) b = P.hi[k];
-            else continue;
-            const double t = __ddiv_rn(__dadd_rn(b, -X[k]), dW[k]);
-            if (t < tmin) {
-                tmin = t;
-                kstar = k;
-                bstar = b;
-            }
-        }
-        if (kstar < 0) return kNaN;
-        theta = fmin(fmax(tmin, 0.0), 1.0);
-        for (int k = 0; k < 3; ++k) xs[k] = __dadd_rn(X[k], __dmul_rn(theta, dW[k]));
-        xs[kstar] = bstar;
-        face = 2 * kstar + (bstar == P.hi[kstar] ? 1 : 0);
-    } else {
-        xs[0] = Y[0];
-        xs[1] = Y[1];
-        xs[2] = Y[2];
-    }
-    const double r = rho_f64(P, M, xs);
-    I = __dadd_rn(I, __dmul_rn(__dmul_rn(__dmul_rn(0.5, __dadd_rn(rp, r)), theta), P.dt));
-    return __dadd_rn(boundary_value(P, M, face, xs), -__dmul_rn(P.two_pi_G, I));
 }
 
 // Mixed walk exit (run by exit_mixed_kernel, one thread per path, so the
@@ -264,16 +136,6 @@ __device__ __forceinline__ void put_exit(const WalkParams& P, int c, unsigned lo
     r[1] = make_float4(y1, y2, __int_as_float(__double2loint(acc)), __int_as_float(__double2hiint(acc)));
 }
 
-// A density that is rho0 or 0: its source sum is rho0 times a count of
-// points, kept exactly (a single-precision count of whole and half points in
-// registers, half points as a 64-bit integer beyond it), so no double
-// precision is needed before the exit and the sum does not depend on the
-// order of its terms.
-template <int RHO>
-constexpr bool kTwoValued = RHO == MCG_RHO_PRISM || RHO == MCG_RHO_SPHERE;
-template <int RHO>
-constexpr bool kVoxel = RHO == MCG_RHO_VOXEL || RHO == kRhoVoxelPacked;
-
 // Source sum of a copy: `held` is the flushed part (a double's bits, or a
 // count of half points), `part` the single-precision part since.
 template <int RHO>
@@ -293,47 +155,6 @@ __device__ __forceinline__ unsigned long long flushed(unsigned long long held, f
         return held + (unsigned long long)(2.0f * part);
     else
         return (unsigned long long)__double_as_longlong(__longlong_as_double((long long)held) + (double)part);
-}
-
-__device__ __forceinline__ void write_path(const WalkParams& P, int32_t* status, unsigned long long item, double u0,
-                                           double up, double um, int64_t steps)
-{
-    const double d = P.crn ? (up - um) / (2.0 * P.h) : kNaN;
-    P.pp_u[item] = u0;
-    P.pp_d[item] = d;
-    P.pp_steps[item] = steps;
-    const bool bad = !isfinite(u0) || (P.crn && !isfinite(d));
-    if (bad) atomicOr(status, 1 << MCG_ERR_NONFINITE);
-}
-
-// ---------------------------------------------------------------------------
-// Brownian-bridge exit test of an inside step X -> Y (the paper's Remark on
-// exit-time estimation, after Gobet): the bridge crosses the plane of a face
-// at distances d_X, d_Y with probability exp(-2 d_X d_Y / sd^2); with the
-// faces taken as independent the step exits with probability
-// 1 - prod (1 - p_face).  One uniform per RNG-step n: Philox counter
-// (n / 4, p, s, 2), word n % 4, shared by the copies.  Returns the face with
-// the largest p (2k lower, 2k+1 upper) if the step exits, else -1.
-// ---------------------------------------------------------------------------
-__device__ __noinline__ int bridge_face_f64(const WalkParams& P, const double* X, const double* Y, uint32_t s,
-                                            uint32_t p, uint32_t n)
-{
-    double q = 1.0, pmax = -1.0;
-    int kmax = -1;
-    for (int f = 0; f < 6; ++f) {
-        const int k = f >> 1;
-        const double dX = (f & 1) ? __dadd_rn(P.hi[k], -X[k]) : __dadd_rn(X[k], -P.lo[k]);
-        const double dY = (f & 1) ? __dadd_rn(P.hi[k], -Y[k]) : __dadd_rn(Y[k], -P.lo[k]);
-        const double pk = exp(__ddiv_rn(__dmul_rn(__dmul_rn(-2.0, dX), dY), __dmul_rn(P.sd, P.sd)));
-        q = __dmul_rn(q, __dadd_rn(1.0, -pk));
-        if (pk > pmax) {
-            pmax = pk;
-            kmax = f;
-        }
-    }
-    const uint4 w = philox4x32_10(make_uint4(n >> 2, p, s, 2u), P.key0, P.key1);
-    const uint32_t word = (n & 3u) == 0u ? w.x : (n & 3u) == 1u ? w.y : (n & 3u) == 2u ? w.z : w.w;
-    return (u01_f64(word) < 1.0 - q) ? kmax : -1;
 }
 
 // Single-precision bridge test of the copies `cand` for step m of block blk
@@ -383,132 +204,6 @@ __device__ __noinline__ unsigned bridge_exits_f32(const WalkParams& P, unsigned 
 }
 
 // ---------------------------------------------------------------------------
-// Plain double-precision walk.
-// ---------------------------------------------------------------------------
-template <bool CRN, bool SEG>
-__global__ void __launch_bounds__(128) walk_fp64_kernel(const WalkParams P)
-{
-    constexpr int NC = CRN ? 3 : 1;
-    bool busy = false, drained = false;
-    unsigned long long item = 0ull;
-    uint32_t s = 0u, p = 0u;
-    int64_t n = 0;
-    double W[3], I[NC], rp[NC], u[3];
-    unsigned alive = 0u;
-    int64_t steps = 0;
-    const double off[3] = {0.0, P.h, -P.h};
-    unsigned iter = 0u;
-    // the walk's request (its own in a multi-request launch)
-    uint32_t k0 = P.key0, k1 = P.key1;
-    int32_t* status = P.status;
-    ModelRef M = model_of(P);
-
-    for (;;) {
-        if ((++iter & 255u) == 0u && cancelled(P)) {
-            if ((threadIdx.x & 31) == 0) atomicOr(P.status, 1 << MCG_ERR_CANCELLED);
-            if (busy) {  // this walk gives no result
-                P.pp_u[item] = kNaN;
-                P.pp_d[item] = kNaN;
-                P.pp_steps[item] = steps;
-            }
-            busy = false;
-            drained = true;
-        }
-        unsigned long long next = 0ull;
-        if (refill(P, busy, 32u, drained, next)) {
-            item = next;
-            const double* st = P.stations;
-            unsigned long long local = item, N = (unsigned long long)P.N, p0 = (unsigned long long)P.p0;
-            if constexpr (SEG) {
-                const WalkSeg& g = P.seg[find_seg(P, item)];
-                local = item - g.begin;
-                N = (unsigned long long)g.N;
-                p0 = (unsigned long long)g.p0;
-                st = g.stations;
-                status = g.status;
-                k0 = g.key0;
-                k1 = g.key1;
-                M = model_of(g);
-            }
-            s = (uint32_t)(local / N);
-            if (station_ok(P, st, status, s, item)) {
-                p = (uint32_t)(p0 + local % N);
-                for (int k = 0; k < 3; ++k) W[k] = st[3 * s + k];
-                for (int c = 0; c < NC; ++c) {
-                    const double X[3] = {W[0], W[1], __dadd_rn(W[2], off[c])};
-                    rp[c] = rho_f64(P, M, X);
-                    I[c] = 0.0;
-                }
-                u[0] = u[1] = u[2] = kNaN;
-                alive = (1u << NC) - 1u;
-                n = 0;
-                steps = 0;
-                busy = true;
-            }
-        }
-        if (!__any_sync(kFull, busy)) break;
-        if (!busy) continue;
-
-        double z[12];
-        normals12_f64(s, p, (uint32_t)(n >> 2), k0, k1, z);
-#pragma unroll 1
-        for (int m = 0; m < 4 && alive; ++m) {
-            const double dW[3] = {__dmul_rn(P.sd, z[3 * m]), __dmul_rn(P.sd, z[3 * m + 1]),
-                                  __dmul_rn(P.sd, z[3 * m + 2])};
-            const double Wn[3] = {__dadd_rn(W[0], dW[0]), __dadd_rn(W[1], dW[1]), __dadd_rn(W[2], dW[2])};
-#pragma unroll
-            for (int c = 0; c < NC; ++c) {
-                if (!(alive & (1u << c))) continue;
-                const double X[3] = {W[0], W[1], __dadd_rn(W[2], off[c])};
-                const double Y[3] = {Wn[0], Wn[1], __dadd_rn(Wn[2], off[c])};
-                steps += 1;
-                bool inside;
-                if (P.ball) {
-                    const double dx = __dadd_rn(Y[0], -P.cen[0]), dy = __dadd_rn(Y[1], -P.cen[1]),
-                                 dz = __dadd_rn(Y[2], -P.cen[2]);
-                    inside = __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz)) < P.R2;
-                } else {
-                    inside = Y[0] > P.lo[0] && Y[0] < P.hi[0] && Y[1] > P.lo[1] && Y[1] < P.hi[1] && Y[2] > P.lo[2] &&
-                             Y[2] < P.hi[2];
-                }
-                // (multi-request launches run without the bridge test)
-                const int kb = (!SEG && inside && P.bridge) ? bridge_face_f64(P, X, Y, s, p, (uint32_t)n) : -1;
-                if (inside && kb < 0) {
-                    const double r = rho_f64(P, M, Y);
-                    I[c] = __dadd_rn(I[c], __dmul_rn(__dmul_rn(0.5, __dadd_rn(rp[c], r)), P.dt));
-                    rp[c] = r;
-                } else if (inside) {
-                    // the bridge left Omega: end on face kb below Y after a full step
-                    double xs[3] = {Y[0], Y[1], Y[2]};
-                    xs[kb >> 1] = (kb & 1) ? P.hi[kb >> 1] : P.lo[kb >> 1];
-                    const double r = rho_f64(P, M, xs);
-                    const double Ic = __dadd_rn(I[c], __dmul_rn(__dmul_rn(0.5, __dadd_rn(rp[c], r)), P.dt));
-                    u[c] = __dadd_rn(boundary_value(P, M, kb, xs), -__dmul_rn(P.two_pi_G, Ic));
-                    alive &= ~(1u << c);
-                } else {
-                    u[c] = exit_fp64(P, M, X, dW, Y, I[c], rp[c]);
-                    alive &= ~(1u << c);
-                }
-            }
-            W[0] = Wn[0];
-            W[1] = Wn[1];
-            W[2] = Wn[2];
-            ++n;
-        }
-        if (!alive) {
-            write_path(P, status, item, u[0], u[1], u[2], steps);
-            busy = false;
-        } else if (n >= P.max_steps) {
-            atomicOr(status, 1 << MCG_ERR_STEP_CAP);
-            P.pp_u[item] = kNaN;
-            P.pp_d[item] = kNaN;
-            P.pp_steps[item] = steps;
-            busy = false;
-        }
-    }
-}
-
-// ---------------------------------------------------------------------------
 // Mixed-precision walk: single-precision stepping and no double-precision
 // arithmetic in the step loop.  A warp works in one of two ways:
 //
@@ -535,28 +230,6 @@ __global__ void __launch_bounds__(128) walk_fp64_kernel(const WalkParams P)
 // ---------------------------------------------------------------------------
 constexpr unsigned kStripMax = 16;
 constexpr int kStripRow = 33;  // float4 per row: rows of one block column fall into different banks
-
-// Conservative tests of a four-step block.  No coordinate moves by more than -(nr[0] + ... + nr[5]) over the
-// block, so if that bound keeps every copy inside the conservative box
-// (ball) -- `inside` -- the block needs no exit test, and if it also stays
-// outside the density's support box -- `quiet` -- only the position changes.
-// The boxes' margin, 1e-5 of the domain, is some twenty times the
-// single-precision rounding of the bound and of the four moves.
-template <int RHO, bool BALL>
-__device__ __forceinline__ void block_bounds(const WalkParams& P, float x, float y, float z, const float nr[6],
-                                             bool& inside, bool& quiet)
-{
-    const float rs = ((nr[0] + nr[1]) + (nr[2] + nr[3])) + (nr[4] + nr[5]);  // <= 0
-    const float ax = fabsf(x) - rs, ay = fabsf(y) - rs, az = fabsf(z) - rs;
-    if (BALL) inside = fmaf(ax, ax, fmaf(ay, ay, az * az)) < P.in_r2_f;
-    else inside = ax < P.in_f[0] && ay < P.in_f[1] && az < P.in_f[2];
-    quiet = inside;
-    if constexpr (kTwoValued<RHO>)
-        quiet = inside && (fabsf(x - P.far_c[0]) + rs > P.far_h[0] || fabsf(y - P.far_c[1]) + rs > P.far_h[1] ||
-                           fabsf(z - P.far_c[2]) + rs > P.far_h[2]);
-    else if constexpr (kVoxel<RHO>)
-        quiet = false;
-}
 
 // Copies strictly inside Omega at the walk position (x, y, z): bit c for copy c.
 template <bool CRN, bool BALL>
@@ -1286,10 +959,7 @@ const void* mixed_fn(bool crn, bool seg)
 
 const void* kernel_fn(int precision, int rho_kind, bool crn, bool seg)
 {
-    if (precision == MCG_FP64) {
-        if (seg) return crn ? (const void*)walk_fp64_kernel<true, true> : (const void*)walk_fp64_kernel<false, true>;
-        return crn ? (const void*)walk_fp64_kernel<true, false> : (const void*)walk_fp64_kernel<false, false>;
-    }
+    if (precision == MCG_FP64) return walk64_fn(rho_kind, crn, seg);
     switch (rho_kind) {
     case kRhoVoxelPacked: return mixed_fn<kRhoVoxelPacked>(crn, seg);
     case MCG_RHO_SPHERE: return mixed_fn<MCG_RHO_SPHERE>(crn, seg);
@@ -1329,10 +999,7 @@ void touch_mixed()
 
 void preload_walk_kernels()
 {
-    touch(walk_fp64_kernel<true, false>);
-    touch(walk_fp64_kernel<false, false>);
-    touch(walk_fp64_kernel<true, true>);
-    touch(walk_fp64_kernel<false, true>);
+    preload_walk64_kernels();
     touch_mixed<MCG_RHO_NONE>();
     touch_mixed<MCG_RHO_SPHERE>();
     touch_mixed<MCG_RHO_PRISM>();
@@ -1361,8 +1028,9 @@ cudaError_t launch_walk(const WalkParams& P0, int precision, int block, cudaStre
     const int per_sm = walk_blocks_per_sm(precision, kind, block, P.seg != nullptr);
     long long grid = (long long)sms * per_sm;
     const long long need = (long long)((P.total + (unsigned long long)block - 1ull) / (unsigned long long)block);
+    if (precision == MCG_FP64) return launch_walk64(P, block, (int)grid, st);
     P.quota = 32;
-    if (precision == MCG_MIXED) {
+    {
         // Walks per warp.  With a warpful for every resident warp the lanes
         // run a walk each; with fewer the walks are spread over all warps,
         // up to kStripMax each, which run them as strips.  Where the line
@@ -1381,21 +1049,8 @@ cudaError_t launch_walk(const WalkParams& P0, int precision, int block, cudaStre
         } else if (grid > need) {
             grid = need;
         }
-    } else if (grid > need) {
-        grid = need > 0 ? need : 1;
     }
     if (grid < 1) grid = 1;
-    const bool crn = P.crn != 0;
-    if (precision == MCG_FP64) {
-        if (P.seg) {
-            if (crn) walk_fp64_kernel<true, true><<<(int)grid, block, 0, st>>>(P);
-            else walk_fp64_kernel<false, true><<<(int)grid, block, 0, st>>>(P);
-        } else {
-            if (crn) walk_fp64_kernel<true, false><<<(int)grid, block, 0, st>>>(P);
-            else walk_fp64_kernel<false, false><<<(int)grid, block, 0, st>>>(P);
-        }
-        return cudaGetLastError();
-    }
     switch (kind) {
     case kRhoVoxelPacked: return launch_mixed_rho<kRhoVoxelPacked>(P, block, (int)grid, st);
     case MCG_RHO_SPHERE: return launch_mixed_rho<MCG_RHO_SPHERE>(P, block, (int)grid, st);

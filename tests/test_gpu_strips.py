@@ -1,7 +1,8 @@
-"""A walk gives the same numbers whether a lane steps it alone (a launch that
-fills the GPU) or the lanes of a warp share it (a launch of few walks): the
-same paths from both, over the densities, domains and options of the mixed
-walk, path counts that leave ragged groups, and step caps inside a block."""
+"""A walk gives the same numbers however many lanes run it: a lane alone (the
+mixed walk in a launch that fills the GPU), four lanes (the double-precision
+walk there), or all the lanes of a warp (a launch of few walks).  The same
+paths from both, over the densities, domains and options of either walk, path
+counts that leave ragged groups, and step caps inside a block."""
 import numpy as np
 import pytest
 import torch
@@ -14,7 +15,8 @@ from paper_1709_07469_gb300.device import DeviceSolve
 from tests.helpers import smooth_tables
 
 pytestmark = pytest.mark.gpu
-FULL = 200_000  # walks that fill every lane of the GPU
+FULL = {M.MCG_MIXED: 200_000, M.MCG_FP64: 20_000}  # walks that fill the GPU
+BOTH = pytest.mark.parametrize("precision", [M.MCG_MIXED, M.MCG_FP64])
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -23,8 +25,8 @@ def lib():
     M.load()
 
 
-def per_path(w, st, N, cap=None, **kw):
-    ds = DeviceSolve(w, stations=st, batch=N, precision=M.MCG_MIXED, **kw)
+def per_path(w, st, N, cap, **kw):
+    ds = DeviceSolve(w, stations=st, batch=N, **kw)
     if cap:
         ds.opts.max_steps = cap
     ds.reset()
@@ -32,10 +34,10 @@ def per_path(w, st, N, cap=None, **kw):
     return (*ds.per_path(), int(ds.status[0].item()))
 
 
-def same_paths(w, few, cap=None, rounding=0.0, **kw):
+def same_paths(w, few, precision, cap=None, rounding=0.0, **kw):
     st = w.stations[:2]
-    a = per_path(w, st, few, cap, **kw)
-    b = per_path(w, st, FULL // 2, cap, **kw)
+    a = per_path(w, st, few, cap, precision=precision, **kw)
+    b = per_path(w, st, FULL[precision] // 2, cap, precision=precision, **kw)
     assert a[3] == b[3]
     assert np.array_equal(a[2], b[2][:, :few])
     for x, y in zip(a[:2], b[:2]):
@@ -60,25 +62,30 @@ CASES = {
 }
 
 
+@BOTH
 @pytest.mark.parametrize("few", [1, 5, 33, 1001])
 @pytest.mark.parametrize("name", CASES)
-def test_shared_walks_equal_lone_ones(name, few):
-    same_paths(CASES[name], few)
+def test_shared_walks_equal_lone_ones(name, few, precision):
+    same_paths(CASES[name], few, precision)
 
 
+@BOTH
 @pytest.mark.parametrize("cap", [1, 6, 127, 130])
-def test_step_cap_inside_a_shared_round(cap):
-    same_paths(SPHERE.with_(dt=4e-3), 9, cap=cap)
+def test_step_cap_inside_a_shared_round(cap, precision):
+    same_paths(SPHERE.with_(dt=4e-3), 9, precision, cap=cap)
 
 
-@pytest.mark.parametrize("pack", [True, False])
+@pytest.mark.parametrize("precision,pack", [(M.MCG_MIXED, True), (M.MCG_MIXED, False), (M.MCG_FP64, False)])
 @pytest.mark.parametrize("few", [1, 7, 300])
-def test_shared_walks_voxel(few, pack):
+def test_shared_walks_voxel(few, precision, pack):
     """Single-precision partial sums: the flush points of a lane's walk follow
     its warp's refills, so u may differ by the rounding of one flush, at most
     64 * 2^-24 ~ 4e-6 of the source integral, which is below max |u| here (and
-    u by 1 / h of that in the centred difference, h = 1)."""
+    u by 1 / h of that in the centred difference, h = 1).  The double-precision
+    walk's sums are added per lane, then over the lanes: up to 4000 terms in
+    another order, 4000 * 2^-53 < 1e-12."""
     w = W.voxel_survey(shape=(32, 32, 16), table_n=(33, 33), step=20.0)
     grid = torch.from_numpy(oracle.grf_density(1, 32, 32, 16, sigma_vox=2.0, amp=300.0)).cuda()
     faces = torch.from_numpy(smooth_tables(w, scale=-1e-4)).cuda()
-    same_paths(w, few, rounding=4e-6, grid=grid, faces=faces, pack=pack)
+    rounding = 4e-6 if precision == M.MCG_MIXED else 1e-12
+    same_paths(w, few, precision, rounding=rounding, grid=grid, faces=faces, pack=pack)
