@@ -217,7 +217,9 @@ MCG_API const char* mcg_version(void);
  *            are copied into the call's workspace; the device-level entry
  *            points below take device pointers only).
  *   out      : HOST arrays of length S.
- * Blocking.  Allocates a device workspace for the duration of the call:
+ * Blocking.  Takes a device workspace for the duration of the call from a
+ * memory pool of the library's own (which keeps up to 256 MiB per device for
+ * later calls and hands back the rest):
  * mcg_workspace_bytes(S, batch), plus the packed copies of a voxel grid and
  * of boundary tables (mcg_voxel_pack_bytes, mcg_table_pack_bytes) unless the
  * caller passes them, plus the grid and tables themselves when they are in

@@ -126,6 +126,7 @@ size_t solve_set_bytes(int64_t S, int64_t batch);
 cudaError_t reset_walk(const WalkParams& P, cudaStream_t st);
 
 // Kernel launchers (mcg_walk.cu).
+cudaError_t launch_reset(const WalkParams& P, cudaStream_t st);
 cudaError_t launch_walk(const WalkParams& P, int precision, int block, cudaStream_t st);
 int walk_blocks_per_sm(int precision, int rho_kind, int block, bool seg = false);
 // The double-precision walk (mcg_walk64.cu): its kernel, and its launch on at

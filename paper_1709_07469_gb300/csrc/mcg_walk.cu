@@ -919,6 +919,25 @@ __global__ void __launch_bounds__(128) exit_mixed_kernel(const WalkParams P)
     if (lane < qn) exit_item<RHO, SEG>(P, q[lane], hf);
 }
 
+// Before a walk: the work counter at zero, and no item with a result that an
+// earlier launch left: steps 0, which also clears the mixed walk's completion
+// flags (its exit kernel writes NaN for items without one), and NaN per-path
+// values for the double-precision walk, which writes them directly.  One
+// launch (as memsets the four took 4 us each of a small solve).
+__global__ void __launch_bounds__(256) reset_kernel(unsigned long long* counter, int64_t* steps, double* u, double* d,
+                                                    unsigned long long n)
+{
+    const unsigned long long first = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (first == 0ull) *counter = 0ull;
+    for (unsigned long long i = first; i < n; i += (unsigned long long)gridDim.x * blockDim.x) {
+        steps[i] = 0;
+        if (u) {
+            u[i] = kNaN;
+            d[i] = kNaN;
+        }
+    }
+}
+
 template <int RHO, bool CRN, bool BRIDGE, bool BALL, bool SEG>
 cudaError_t launch_mixed(const WalkParams& P, int block, int grid, cudaStream_t st)
 {
@@ -997,8 +1016,17 @@ void touch_mixed()
 
 }  // namespace
 
+cudaError_t launch_reset(const WalkParams& P, cudaStream_t st)
+{
+    const unsigned long long blocks = (P.total + 1023ull) / 1024ull;
+    reset_kernel<<<(unsigned)(blocks < 1ull ? 1ull : blocks < 1216ull ? blocks : 1216ull), 256, 0, st>>>(
+        P.counter, P.pp_steps, P.frec ? nullptr : P.pp_u, P.frec ? nullptr : P.pp_d, P.total);
+    return cudaGetLastError();
+}
+
 void preload_walk_kernels()
 {
+    touch(reset_kernel);
     preload_walk64_kernels();
     touch_mixed<MCG_RHO_NONE>();
     touch_mixed<MCG_RHO_SPHERE>();
