@@ -222,11 +222,11 @@ __device__ __noinline__ unsigned bridge_exits_f32(const WalkParams& P, unsigned 
 // Both take the same steps in the same arithmetic, so a walk's numbers do not
 // depend on how it was run.  What bounds them, on the prism ore body (1 m
 // steps): a walk alone takes 115 ns a step as a lane (the block's dependent
-// generator, logarithm and root, ~950 cycles) and 10 ns as a strip of 32 (that
+// generator, logarithm and root, ~950 cycles) and 7 ns as a strip of 32 (that
 // once per 32 blocks, and the chain, 16 cycles a block); with the GPU full,
-// lanes run 340 steps/ns, strips 240 (k = 2) to 100 (k = 32), as the chain
+// lanes run 340 steps/ns, strips 240 (k = 2) to 190 (k = 16), as the chain
 // idles most lanes, so a full warp runs lanes.  Solves that this shortens:
-// 30 x 256 paths 168 -> 18 ms, 30 x 8192 paths 317 -> 155 ms.
+// 30 x 256 paths 168 -> 15 ms, 30 x 8192 paths 317 -> 154 ms.
 // ---------------------------------------------------------------------------
 constexpr unsigned kStripMax = 16;
 constexpr int kStripRow = 33;  // float4 per row: rows of one block column fall into different banks
@@ -269,6 +269,23 @@ __device__ __forceinline__ void bridge_point(const WalkParams& P, int c, int f, 
     else out[2] = b;
 }
 
+// The moves of block `blk` of walk (s, p) to column `lane` of the strip:
+// per coordinate four steps to a float4, radii in rows 0-2, cosines or sines
+// in rows 3-5.  Returns minus the sum of the radii.
+__device__ __forceinline__ float strip_moves(float4* strip, int lane, uint32_t s, uint32_t p, uint32_t blk, uint32_t k0,
+                                             uint32_t k1, float lnscale)
+{
+    float nr[6], cs[12];
+    polar12_f32(s, p, blk, k0, k1, lnscale, nr, cs);
+    strip[0 * kStripRow + lane] = make_float4(nr[0], nr[1], nr[3], nr[4]);
+    strip[1 * kStripRow + lane] = make_float4(nr[0], nr[2], nr[3], nr[5]);
+    strip[2 * kStripRow + lane] = make_float4(nr[1], nr[2], nr[4], nr[5]);
+    strip[3 * kStripRow + lane] = make_float4(cs[0], cs[3], cs[6], cs[9]);
+    strip[4 * kStripRow + lane] = make_float4(cs[1], cs[4], cs[7], cs[10]);
+    strip[5 * kStripRow + lane] = make_float4(cs[2], cs[5], cs[8], cs[11]);
+    return ((nr[0] + nr[1]) + (nr[2] + nr[3])) + (nr[4] + nr[5]);
+}
+
 // SEG: a multi-request launch (the segment table maps each item to its
 // request); each lane then carries its walk's generator key and model array,
 // and keeps the segment index with the walk's other cold state.
@@ -284,10 +301,11 @@ __global__ void __launch_bounds__(128, MCG_MIXED_MINB) walk_mixed_kernel(const W
     __shared__ unsigned long long sh_item[128];    // work item of the walk
     __shared__ unsigned long long sh_steps[128];   // EM steps of the copies that have exited
     __shared__ int sh_seg[SEG ? 128 : 1];          // segment of the walk (multi-request launch)
-    // strips: the blocks' increments, then positions, then densities; the
-    // walks' positions; per copy the counts (two-valued) or the running sums
+    // strips: the blocks' increments, then densities; the walks' positions and
+    // the blocks' last ones; per copy the counts (two-valued) or running sums
     __shared__ float4 sh_strip[4][6 * kStripRow];
     __shared__ float sh_base[4][3 * kStripMax];
+    __shared__ float sh_end[4][3 * kStripRow];
     using Part = std::conditional_t<kTwoValued<RHO>, unsigned, float>;  // half points, or a running sum
     __shared__ Part sh_part[RHO == MCG_RHO_NONE ? 1 : 3][128];
     __shared__ int sh_own[4][kStripMax];  // slot of the g-th live walk
@@ -393,11 +411,11 @@ __global__ void __launch_bounds__(128, MCG_MIXED_MINB) walk_mixed_kernel(const W
             // Strips.  Group g of k lanes runs the g-th live walk; what the
             // group's lanes share is held alike in all of them.
             // ----------------------------------------------------------------
-            const int G = __popc(livem), k = 32 / G;
+            const int G = __popc(livem), k = 32 / G, ks = k;
             const int g = lane / k < G ? lane / k : G - 1;
             const bool mine = lane / k < G;          // this lane belongs to a group
             const int l = lane - g * k;              // its block of the group's round
-            float4* strip = sh_strip[t >> 5];
+            float4* const strip = sh_strip[t >> 5];
             float* base = sh_base[t >> 5];
             const int* own = sh_own[t >> 5];
             const int rank = __popc(livem & lanes_below);
@@ -442,83 +460,123 @@ __global__ void __launch_bounds__(128, MCG_MIXED_MINB) walk_mixed_kernel(const W
             const uint32_t flushed_at = gblk;  // (the last regrouping)
             // the block at whose end a live walk has reached the step cap
             const int64_t cap_blk = (P.max_steps + 3) / 4;
+            const bool near_cap = __any_sync(kFull, (int64_t)gblk + 16 * k >= cap_blk);
             bool ended = false;  // the group's walk is complete or capped
+            // The chain of one coordinate of a walk from x, the four positions
+            // of each block in the place of its radii; two blocks at a time,
+            // the next two loaded meanwhile.
+            auto run_chain = [&](int q, float x) {
+                float4* rr = strip + (q % 3) * kStripRow + (q / 3) * k;
+                const float4* cc = rr + 3 * kStripRow;
+                auto four = [&x](const float4& a, const float4& b) {
+                    float4 y;
+                    x = y.x = fmaf(a.x, b.x, x);
+                    x = y.y = fmaf(a.y, b.y, x);
+                    x = y.z = fmaf(a.z, b.z, x);
+                    x = y.w = fmaf(a.w, b.w, x);
+                    return y;
+                };
+                float4 a0 = rr[0], b0 = cc[0], a1 = rr[1], b1 = cc[1];  // k >= 2
+                int i = 0;
+#pragma unroll 2
+                for (; i + 4 <= k; i += 2) {
+                    const float4 a2 = rr[i + 2], b2 = cc[i + 2], a3 = rr[i + 3], b3 = cc[i + 3];
+                    rr[i] = four(a0, b0);
+                    rr[i + 1] = four(a1, b1);
+                    a0 = a2;
+                    b0 = b2;
+                    a1 = a3;
+                    b1 = b3;
+                }
+                rr[i] = four(a0, b0);
+                rr[i + 1] = four(a1, b1);
+                if (i + 2 < k) rr[i + 2] = four(rr[i + 2], cc[i + 2]);  // k odd
+            };
+            // A lone walk waits for its chain: only each block's last position
+            // is left (its lane repeats the four moves), as a store of all four
+            // holds the registers of its operands, and the operands are
+            // loaded three blocks ahead.  With the rounds compiled for it alone,
+            // 7.2 ns a step against 9.8.
+            auto run_lone_chain = [&](float x) {
+                const float4 *rr = strip + lane * kStripRow, *cc = rr + 3 * kStripRow;
+                float* e = sh_end[t >> 5] + lane * kStripRow;
+                float4 a[3], b[3];
+#pragma unroll
+                for (int j = 0; j < 3; ++j) {
+                    a[j] = rr[j];
+                    b[j] = cc[j];
+                }
+#pragma unroll
+                for (int i = 0; i < 32; ++i) {
+                    const float4 &u = a[i % 3], &v = b[i % 3];
+                    e[i] = x = fmaf(u.w, v.w, fmaf(u.z, v.z, fmaf(u.y, v.y, fmaf(u.x, v.x, x))));
+                    if (i + 3 < 32) {
+                        a[i % 3] = rr[i + 3];
+                        b[i % 3] = cc[i + 3];
+                    }
+                }
+            };
+            // (compiled twice: for a lone walk, and for several)
+            auto rounds = [&](auto lone) {
             for (int r = 0; r < 16; ++r) {
                 // blocks of this round: up to k, not past the cap, and for a
                 // density that is summed in single precision not past the
                 // next flush (16 blocks after the last)
+                constexpr bool LONE = decltype(lone)::value;
+                const int k = LONE ? 32 : ks;
                 int kk = k;
                 if constexpr (kVoxel<RHO>) kk = min(kk, 16 - (int)((gblk - flushed_at) & 15u));
                 if ((int64_t)gblk + kk > cap_blk) kk = (int)(cap_blk - (int64_t)gblk);
                 const bool act = mine && l < kk;
-                float nr[6], cs[12];
-                polar12_f32(gs, gp, gblk + (uint32_t)l, SEG ? gk0 : P.key0, SEG ? gk1 : P.key1, P.lnscale_f, nr, cs);
-                // the moves per coordinate, four steps to a float4: radii in
-                // rows 0-2, cosines or sines in rows 3-5
-                strip[0 * kStripRow + lane] = make_float4(nr[0], nr[1], nr[3], nr[4]);
-                strip[1 * kStripRow + lane] = make_float4(nr[0], nr[2], nr[3], nr[5]);
-                strip[2 * kStripRow + lane] = make_float4(nr[1], nr[2], nr[4], nr[5]);
-                strip[3 * kStripRow + lane] = make_float4(cs[0], cs[3], cs[6], cs[9]);
-                strip[4 * kStripRow + lane] = make_float4(cs[1], cs[4], cs[7], cs[10]);
-                strip[5 * kStripRow + lane] = make_float4(cs[2], cs[5], cs[8], cs[11]);
+                const float rs = strip_moves(strip, lane, gs, gp, gblk + (uint32_t)l, SEG ? gk0 : P.key0,
+                                             SEG ? gk1 : P.key1, P.lnscale_f);
                 __syncwarp();
-                float4 w0 = make_float4(base[3 * g], base[3 * g + 1], base[3 * g + 2], 0.f);  // before the round
-                // the chain of positions: lane q runs coordinate q % 3 of walk
-                // q / 3 and leaves the four positions of each block in rows 0-2
-                for (int q = lane; q < 3 * G; q += 32) {
-                    float x = base[q];
-                    float4* rr = strip + (q % 3) * kStripRow + (q / 3) * k;
-                    const float4* cc = rr + 3 * kStripRow;
-                    auto four = [&x](const float4& a, const float4& b) {
-                        float4 y;
-                        x = y.x = fmaf(a.x, b.x, x);
-                        x = y.y = fmaf(a.y, b.y, x);
-                        x = y.z = fmaf(a.z, b.z, x);
-                        x = y.w = fmaf(a.w, b.w, x);
-                        return y;
+                const float3 w0 = make_float3(base[3 * g], base[3 * g + 1], base[3 * g + 2]);  // before the round
+                if constexpr (LONE) {
+                    if (lane < 3) run_lone_chain(base[lane]);
+                } else {
+                    for (int q = lane; q < 3 * G; q += 32) run_chain(q, base[q]);
+                }
+                __syncwarp();
+                float px[5], py[5], pz[5];
+                if constexpr (LONE) {
+                    const float* e = sh_end[t >> 5];
+                    auto four = [&](int c, float x, float* p) {
+                        const float4 a = strip[c * kStripRow + lane], b = strip[(c + 3) * kStripRow + lane];
+                        p[0] = lane > 0 ? e[c * kStripRow + lane - 1] : x;
+                        p[1] = fmaf(a.x, b.x, p[0]);
+                        p[2] = fmaf(a.y, b.y, p[1]);
+                        p[3] = fmaf(a.z, b.z, p[2]);
+                        p[4] = fmaf(a.w, b.w, p[3]);
                     };
-                    // two blocks at a time, the next two loaded meanwhile
-                    // (32 cycles of arithmetic cover a shared-memory read)
-                    float4 a0 = rr[0], b0 = cc[0], a1 = rr[1], b1 = cc[1];  // k >= 2
-                    int i = 0;
-                    for (; i + 4 <= k; i += 2) {
-                        const float4 a2 = rr[i + 2], b2 = cc[i + 2], a3 = rr[i + 3], b3 = cc[i + 3];
-                        rr[i] = four(a0, b0);
-                        rr[i + 1] = four(a1, b1);
-                        a0 = a2;
-                        b0 = b2;
-                        a1 = a3;
-                        b1 = b3;
-                    }
-                    rr[i] = four(a0, b0);
-                    rr[i + 1] = four(a1, b1);
-                    if (i + 2 < k) rr[i + 2] = four(rr[i + 2], cc[i + 2]);  // k odd
+                    four(0, w0.x, px);
+                    four(1, w0.y, py);
+                    four(2, w0.z, pz);
+                } else {
+                    auto four = [&](int c, float x, float* p) {
+                        const float4 a = strip[c * kStripRow + lane];
+                        const float before = __shfl_up_sync(kFull, a.w, 1);
+                        p[0] = l > 0 ? before : x;
+                        p[1] = a.x;
+                        p[2] = a.y;
+                        p[3] = a.z;
+                        p[4] = a.w;
+                    };
+                    four(0, w0.x, px);
+                    four(1, w0.y, py);
+                    four(2, w0.z, pz);
                 }
-                __syncwarp();
-                const float4 X = strip[0 * kStripRow + lane], Y = strip[1 * kStripRow + lane],
-                             Z = strip[2 * kStripRow + lane];
-                {   // the position before this lane's block
-                    const float x = __shfl_up_sync(kFull, X.w, 1), y = __shfl_up_sync(kFull, Y.w, 1),
-                                z = __shfl_up_sync(kFull, Z.w, 1);
-                    if (l > 0) {
-                        w0.x = x;
-                        w0.y = y;
-                        w0.z = z;
-                    }
-                }
-                __syncwarp();
-                if (act && l == kk - 1) {
-                    base[3 * g] = X.w;
-                    base[3 * g + 1] = Y.w;
-                    base[3 * g + 2] = Z.w;
+                if (act && l == kk - 1) {  // (the others have read it before the chain)
+                    base[3 * g] = px[4];
+                    base[3 * g + 1] = py[4];
+                    base[3 * g + 2] = pz[4];
                 }
                 bool inside, quiet;
-                block_bounds<RHO, BALL>(P, w0.x, w0.y, w0.z, nr, inside, quiet);
-                const bool all_inside = __all_sync(kFull, inside || !act);
-                const bool all_quiet = __all_sync(kFull, quiet || !act);
-                if (!all_quiet) {
-                    const float px[5] = {w0.x, X.x, X.y, X.z, X.w}, py[5] = {w0.y, Y.x, Y.y, Y.z, Y.w},
-                                pz[5] = {w0.z, Z.x, Z.y, Z.z, Z.w};
+                const float reach[6] = {rs, 0.f, 0.f, 0.f, 0.f, 0.f};
+                block_bounds<RHO, BALL>(P, px[0], py[0], pz[0], reach, inside, quiet);
+                bool any_out = false;
+                if (!__all_sync(kFull, quiet || !act)) {
+                    const bool all_inside = __all_sync(kFull, inside || !act);
                     const uint32_t myblk = gblk + (uint32_t)l;
                     unsigned la = act ? gal : 0u;  // copies live at this point of the block
                     unsigned out = 0u;             // copies that leave in this block ...
@@ -565,7 +623,7 @@ __global__ void __launch_bounds__(128, MCG_MIXED_MINB) walk_mixed_kernel(const W
                     }
                     // the first block of the round in which each copy leaves
                     int first[3] = {32, 32, 32};
-                    const bool any_out = __any_sync(kFull, out != 0u);
+                    any_out = __any_sync(kFull, out != 0u);
                     if (any_out) {
 #pragma unroll
                         for (int c = 0; c < NC; ++c) {
@@ -652,6 +710,8 @@ __global__ void __launch_bounds__(128, MCG_MIXED_MINB) walk_mixed_kernel(const W
                         }
                     }
                 }
+                __syncwarp();
+                if (!any_out && !near_cap) continue;
                 if (mine && gal == 0u) {
                     if (l == 0) P.pp_steps[sh_item[slot]] = (long long)(sh_steps[slot] | (unsigned long long)kDoneFlag);
                     ended = true;
@@ -664,9 +724,11 @@ __global__ void __launch_bounds__(128, MCG_MIXED_MINB) walk_mixed_kernel(const W
                     }
                     ended = true;
                 }
-                __syncwarp();
                 if (__any_sync(kFull, ended)) break;  // regroup the others, or take new walks
             }
+            };
+            if (G == 1) rounds(std::true_type{});
+            else rounds(std::false_type{});
             // back to the owners
             if constexpr (kTwoValued<RHO>) add_counts();
             const int from = rank * k & 31;
@@ -1068,7 +1130,8 @@ cudaError_t launch_walk(const WalkParams& P0, int precision, int block, cudaStre
         // precision sums follows the walks that share a warp, and 32
         // consecutive items keep it the same however many SMs there are.
         const long long per_block = block / 32;
-        const long long per_warp = (long long)(P.total / (unsigned long long)(grid * per_block));
+        const unsigned long long warps = (unsigned long long)(grid * per_block);
+        const long long per_warp = (long long)(P.total / warps);
         if (per_warp < 32 && P.rho_kind != MCG_RHO_VOXEL) {
             P.quota = (int32_t)(per_warp < 1 ? 1 : per_warp > (long long)kStripMax ? kStripMax : per_warp);
             const long long spread = (long long)((P.total + (unsigned long long)per_block - 1ull) /
