@@ -332,7 +332,7 @@ MCG_API int mcg_states_merge(const mcg_station_state* parts, int64_t R, int64_t 
 /* mcg_autotune: picks the launch shape of the walk for this problem and
  * writes it into *opts, in two stages timed with CUDA events (one warm-up
  * launch, then the median of three timed launches per candidate):
- *   1. opts->block (64, 96, 128) on short walks of the given stations capped
+ *   1. opts->block (64, 128) on short walks of the given stations capped
  *      at 2048 RNG-steps (the stepping rate, every lane busy; all walks of a
  *      warp end together, so the refill policy plays no part);
  *   2. mixed walk: opts->refill_min (1, 4, 16) on uncapped walks, two per
