@@ -382,7 +382,7 @@ int status_from_bits(int bits)
     if (bits == 0) return MCG_OK;
     if (bits & (1 << MCG_ERR_ARG)) return set_error(MCG_ERR_ARG, "a station lies on or outside the domain");
     if (bits & (1 << MCG_ERR_TIMEOUT))
-        return set_error(MCG_ERR_TIMEOUT, "a bounded wait on a migrated walk gave up (that walk reads NaN)");
+        return set_error(MCG_ERR_TIMEOUT, "a bounded wait for a handed-over walk gave up (that walk reads NaN)");
     if (bits & (1 << MCG_ERR_CANCELLED)) return set_error(MCG_ERR_CANCELLED, "cancelled");
     if (bits & (1 << MCG_ERR_STEP_CAP)) return set_error(MCG_ERR_STEP_CAP, "a path exceeded max_steps");
     if (bits & (1 << MCG_ERR_NONFINITE)) return set_error(MCG_ERR_NONFINITE, "a per-path value was not finite");
@@ -560,7 +560,7 @@ int mcgrav_solve(const mcg_domain* domain, const mcg_density* density, const mcg
 
     int64_t batch = opts.batch_paths;
     if (batch <= 0) {
-        // per-path buffers, exit records and migration pool of at most ~4 GiB per launch
+        // per-path buffers and walk scratch of at most ~4 GiB per launch
         const double per_path = (double)mcg_workspace_bytes(S, 4096) / (4096.0 * (double)S);
         const int64_t cap = (int64_t)((double)(4ull << 30) / (per_path * (double)S));
         batch = paths < cap ? paths : (cap > 0 ? cap : 1);
@@ -586,12 +586,15 @@ int mcgrav_solve(const mcg_domain* domain, const mcg_density* density, const mcg
     char* ws = nullptr;
     cudaStream_t st = (cudaStream_t)opts.stream;
     cudaMemPool_t pool = nullptr;
-    cudaError_t e = solve_pool(&pool);
+    // a blocking call cannot be part of a capture (a pool allocation alone could)
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(st, &cap);
+    if (e == cudaSuccess && cap != cudaStreamCaptureStatusNone) e = cudaErrorStreamCaptureUnsupported;
+    if (e == cudaSuccess) e = solve_pool(&pool);
     if (e == cudaSuccess) e = cudaMallocFromPoolAsync((void**)&ws, bytes, pool, st);
     if (e != cudaSuccess) {
         cudaGetLastError();
-        return set_error(e == cudaErrorMemoryAllocation ? MCG_ERR_OOM : MCG_ERR_CUDA, "workspace of %zu bytes: %s",
-                         bytes, cudaGetErrorString(e));
+        return set_error(MCG_ERR_OOM, "workspace of %zu bytes: %s", bytes, cudaGetErrorString(e));
     }
     const size_t s_ = (size_t)S, n_ = (size_t)S * (size_t)batch;
     char* q = ws;
@@ -891,7 +894,7 @@ int mcg_walk_static(const mcg_domain* domain, const mcg_density* density, const 
     // the counter starts at zero and every item without its completion flag
     // (the step counts are cleared), so that an item that does not finish
     // (cancel) never reads the last call's records left in the shared array;
-    // there is no migration pool here
+    // the failure-detection hook has no flags here
     e = reset_walk(P, st);
     if (e != cudaSuccess) return cuda_fail(e, "walk reset");
     e = launch_walk(P, opts->precision, opts->block ? opts->block : 128, st);
