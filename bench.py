@@ -45,13 +45,13 @@ SM_MAX_MHZ = 2070.0   # used when nvidia-smi reports no maximum SM clock
 # density 13 + trapezoid 3 = 74; per path-step (3 copies) 74 / 3.
 OPS_PER_RNG_STEP = 74.0
 OPS_PER_PATH_STEP = OPS_PER_RNG_STEP / 3.0
-# Double-precision FMA / add / multiply thread-instructions of the plain FP64
-# walk per RNG-step (its Box-Muller transform, step, tests and sums in
-# double precision), counted by ncu (smsp__sass_thread_inst_executed_op_
-# {dfma,dadd,dmul}_pred_on.sum) on 30 x 32768 prism paths capped at 64
-# RNG-steps; the FP64 walk's roofline is this count against the measured DFMA
-# rate.
-FP64_OPS_PER_RNG_STEP = 118.8
+# Double-precision FMA / add / multiply thread-instructions of the FP64 walk
+# per RNG-step (the products that make its increments, the additions that
+# move it; its functions run in integers), counted by ncu (smsp__sass_thread_
+# inst_executed_op_{dfma,dadd,dmul}_pred_on.sum) on 30 x 32768 prism paths
+# capped at 64 RNG-steps; the FP64 walk's roofline is this count against the
+# measured DFMA rate.
+FP64_OPS_PER_RNG_STEP = 9.9
 L2_FLUSH_BYTES = 256 << 20
 # DRAM bytes (read + write) of one walk_mixed_kernel launch per work item,
 # from ncu's dram__bytes_read.sum + dram__bytes_write.sum (one pass) on a
@@ -72,9 +72,9 @@ def parse():
                     help="paths per station per step (131072: the 10^6 paths of the workload in ~8 steps)")
     ap.add_argument("--block", type=int, default=0, help="threads per block of the walk (0: library default)")
     ap.add_argument("--migrate", type=int, default=1, choices=[0, 1],
-                    help="hand the last walks of sparse warps to warps with free lanes (default 1)")
+                    help="the walk option of that name (default 1); without effect on the walk")
     ap.add_argument("--autotune", type=int, default=1, choices=[0, 1],
-                    help="pick block, refill threshold and spill threshold with mcg_autotune first (default 1)")
+                    help="pick block and refill threshold with mcg_autotune first (default 1)")
     ap.add_argument("--cpu-paths", type=int, default=256, help="paths per station in the CPU-oracle sample")
     ap.add_argument("--skip-cpu", action="store_true")
     ap.add_argument("--skip-fp64", action="store_true")
@@ -447,7 +447,7 @@ def measured_peaks(M, achieved):
 
 
 def fp64_roofline(M, path_steps_per_s):
-    """The plain FP64 walk against the GPU's measured DFMA rate (probe kind
+    """The FP64 walk against the GPU's measured DFMA rate (probe kind
     2): its double-precision FMA / add / multiply instructions per second over
     the rate the FP64 pipe sustains on independent DFMAs.  Capped paths keep
     all three copies alive, so RNG-steps = path-steps / 3."""
@@ -455,7 +455,7 @@ def fp64_roofline(M, path_steps_per_s):
     achieved = path_steps_per_s / 3.0 * FP64_OPS_PER_RNG_STEP / 1e12
     return {"bound": "fp64", "achieved": achieved, "peak": rate / 1e12, "unit": "Tlane-op/s",
             "frac": achieved / (rate / 1e12), "ops_per_rng_step": FP64_OPS_PER_RNG_STEP, "probe_s": secs,
-            "kernel": "walk_fp64_kernel<crn>",
+            "kernel": "walk64_kernel<prism, crn>",
             "peak_source": "measured: 8 independent DFMA chains per thread on every SM, CUDA events",
             "ops_source": "ncu DFMA + DADD + DMUL thread-instructions per RNG-step on the capped prism case"}
 
