@@ -239,7 +239,9 @@ __device__ __noinline__ unsigned bridge_exits_f32(const WalkParams& P, unsigned 
 // once per 32 blocks, and the chain, 16 cycles a block); with the GPU full,
 // lanes run 340 steps/ns, strips 240 (k = 2) to 190 (k = 16), as the chain
 // idles most lanes, so a full warp runs lanes.  Solves that this shortens:
-// 30 x 256 paths 168 -> 15 ms, 30 x 8192 paths 317 -> 154 ms.
+// 30 x 256 paths 178 -> 16 ms, 30 x 8192 paths 333 -> 150 ms.  The price: the
+// strips' registers leave a full launch 20 warps per SM instead of 24, 1.6 %
+// where a second stream hides the tail anyway (30 x 131072 paths a step).
 // ---------------------------------------------------------------------------
 constexpr unsigned kStripMax = 16;
 constexpr int kStripRow = 33;  // float4 per row: rows of one block column fall into different banks
