@@ -473,8 +473,7 @@ __global__ void __launch_bounds__(128, MCG_MIXED_MINB) walk_mixed_kernel(const W
                 __syncwarp();
             };
             const uint32_t flushed_at = gblk;  // (the last regrouping)
-            // the block at whose end a live walk has reached the step cap
-            const int64_t cap_blk = (P.max_steps + 3) / 4;
+            const int64_t cap_blk = cap_block(P);
             const bool near_cap = __any_sync(kFull, (int64_t)gblk + 16 * k >= cap_blk);
             bool ended = false;  // the group's walk is complete or capped
             // The chain of one coordinate of a walk from x, the four positions

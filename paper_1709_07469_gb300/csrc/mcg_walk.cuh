@@ -61,6 +61,10 @@ __device__ __forceinline__ bool station_ok(const WalkParams& P, const double* st
 
 __device__ __forceinline__ int64_t nstep_of(uint32_t blk, int m) { return 4 * (int64_t)blk + m + 1; }
 
+// The block at whose end a live walk has reached the step cap (max_steps may be
+// the largest integer: no rounding up by an addition).
+__device__ __forceinline__ int64_t cap_block(const WalkParams& P) { return P.max_steps / 4 + (P.max_steps % 4 != 0); }
+
 // The cancel flag may live in host-mapped or device memory and is written
 // by the host while the kernel runs: read it with a system-scope relaxed
 // load so the write is observed whatever caches the line.

@@ -426,7 +426,7 @@ __global__ void __launch_bounds__(128, 4) walk64_kernel(const WalkParams P, cons
         unsigned gal = w.alive;
         ModelRef M = model_of(P);
         if constexpr (SEG) M = model_of(P.seg[w.seg]);
-        const int64_t cap_blk = (P.max_steps + 3) / 4;
+        const int64_t cap_blk = cap_block(P);
         unsigned n_in[3] = {0u, 0u, 0u};        // this lane's points of the support ...
         double r_in[3] = {0.0, 0.0, 0.0};       // ... or densities, not yet in the walk's sums
         auto add_up = [&]() {
