@@ -31,9 +31,10 @@ __global__ void normals_f64_kernel(uint32_t k0, uint32_t k1, uint32_t s, uint32_
             double r;
             float rf;
             int64_t co, si;
-            fx::polar64(fx::g_tables, q ? w.z : w.x, q ? w.w : w.y, r, rf, co, si);
-            out[12 * i + 4 * j + 2 * q] = __dmul_rn(r, __ll2double_rn(co));
-            out[12 * i + 4 * j + 2 * q + 1] = __dmul_rn(r, __ll2double_rn(si));
+            double c, s;
+            fx::polar64(fx::g_tables, q ? w.z : w.x, q ? w.w : w.y, r, rf, co, si, c, s);
+            out[12 * i + 4 * j + 2 * q] = __dmul_rn(r, c);
+            out[12 * i + 4 * j + 2 * q + 1] = __dmul_rn(r, s);
         }
     }
 }

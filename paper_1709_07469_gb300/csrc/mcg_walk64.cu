@@ -1,14 +1,16 @@
 // mcg_walk64.cu -- the double-precision walk (Sec. 2.3 of the paper, steps 1-4).
 //
-// Every number the problem states is a double, rounded operation by operation
+// Increments, positions and exits are doubles, rounded operation by operation
 // (no contraction), so a path agrees with a plain double-precision evaluation
-// to the last bits of log, sqrt, cos and sin.  GB300 does 1.6 double-precision
-// operations a clock and SM, and a step evaluated that way throughout took
-// 166, 6.6 us for a lane.  What is left of them: the products that
-// make an increment (3 a normal) and the additions that move the walk.  The
-// functions are evaluated in 64-bit integers (mcg_fixed.cuh), and the
-// tests of a point (inside Omega, in the density's support, in which cell) in
-// single precision, with doubles where that is too close to call.
+// to the last bits of log, sqrt, cos and sin; the source integral is a sum over
+// the walk's points (exact counts where the density is rho0 or 0, else lane by
+// lane), closed at the exit.  GB300 does 1.6 double-precision operations a clock
+// and SM, and a step evaluated in doubles throughout took 166, 6.6 us for a
+// lane.  What is left of them: the products that make an increment (3 a normal)
+// and the additions that move the walk.  The functions are evaluated in 64-bit
+// integers (mcg_fixed.cuh), and the tests of a point (inside Omega, in the
+// density's support, in which cell) in single precision, with doubles where that
+// is too close to call.
 //
 // A warp holds G <= 8 walks and k = 32 / G lanes share each: a lane makes the
 // increments of one four-step block, a lane per walk and coordinate adds them
@@ -16,11 +18,11 @@
 //
 // What bounds it: with the GPU full the double-precision pipe (busy 74 % of
 // the time: 64 operations of a block's 3100 instructions a lane) and the
-// integer pipes beside it (issue 57 %): 28.7 steps/ns against 3.2 for the plain
+// integer pipes beside it (issue 57 %): 27.2 steps/ns against 3.2 for the plain
 // evaluation (ore body, capped walks).  With few walks the chain of additions
 // and a block's dependent integers: 110 ns a step for a lone walk (6270
-// before).  Walks of the sphere, 8 x 2000 paths: 17.7 -> 0.88 ms; ore body at
-// 10 m steps, 30 x 256 paths: 106.7 -> 2.0 ms.
+// before).  Walks of the sphere, 8 x 2000 paths: 17.7 -> 0.91 ms; ore body at
+// 10 m steps, 30 x 256 paths: 106.7 -> 2.06 ms.
 #include <cmath>
 
 #include <cuda_runtime.h>
@@ -223,8 +225,9 @@ __device__ __noinline__ void step_of(const fx::Tables& tables, double sd, uint4 
         double rd;
         float rf;
         int64_t co, si;
-        fx::polar64(tables, (j & 2) ? v.z : v.x, (j & 2) ? v.w : v.y, rd, rf, co, si);
-        dW[q] = __dmul_rn(sd, __dmul_rn(rd, __ll2double_rn((j & 1) ? si : co)));
+        double cs, sn;
+        fx::polar64(tables, (j & 2) ? v.z : v.x, (j & 2) ? v.w : v.y, rd, rf, co, si, cs, sn);
+        dW[q] = __dmul_rn(sd, __dmul_rn(rd, (j & 1) ? sn : cs));
     }
 }
 
@@ -476,15 +479,15 @@ __global__ void __launch_bounds__(128, 4) walk64_kernel(const WalkParams P, cons
                     double rd;
                     float rf;
                     int64_t co, si;
-                    fx::polar64(tables, v.x, v.y, rd, rf, co, si);
+                    double cs, sn;
+                    fx::polar64(tables, v.x, v.y, rd, rf, co, si, cs, sn);
                     v.x = v.z;
                     v.y = v.w;
                     rf *= T.sd;
                     reach -= rf;
                     const uint32_t j = 4u * i + 2u * q;  // normals j, j + 1: coordinate j % 3 of step j / 3
-                    put(j, __dmul_rn(P.sd, __dmul_rn(rd, __ll2double_rn(co))), rf * ((float)(int32_t)(co >> 32) * 0x1p-31f));
-                    put(j + 1u, __dmul_rn(P.sd, __dmul_rn(rd, __ll2double_rn(si))),
-                        rf * ((float)(int32_t)(si >> 32) * 0x1p-31f));
+                    put(j, __dmul_rn(P.sd, __dmul_rn(rd, cs)), rf * ((float)(int32_t)(co >> 32) * 0x1p-31f));
+                    put(j + 1u, __dmul_rn(P.sd, __dmul_rn(rd, sn)), rf * ((float)(int32_t)(si >> 32) * 0x1p-31f));
                 }
             }
             double W0[3] = {w.w[0], w.w[1], w.w[2]};  // before the block (of the round, for its first)
