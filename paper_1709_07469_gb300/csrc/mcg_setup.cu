@@ -148,6 +148,10 @@ constexpr int kRowsPerTile = 8;
 // core at three sides and without P_10 (1e-8) one table value in a thousand
 // rounded to its neighbour.
 constexpr double kCoreSides = 4.0, kExactSides = 2.0;
+// Beyond 2048 sides P_4 .. P_10 add less than 1e-15 of the cell's term (0.015 y^4,
+// below the pairs' 3e-14), and powers of coordinates counted in sides overflow
+// from 1.6e4 sides on (inf times an underflown y^20 is no number).
+constexpr float kSeriesEnds = 1.0f / 2048.0f;
 
 __device__ __forceinline__ void node_position(const TableParams& T, int64_t node, double x[3])
 {
@@ -303,10 +307,13 @@ __global__ void __launch_bounds__(kTableThreads, 2) tables_kernel(const TablePar
                     Pair y2, P2, y5;
                     const Pair y = rsqrt_pair(pair_of(d2 * inv2), y2);
                     const Pair v = series_second(p2x, c2, X, y, y2, P2, y5);
-                    float P4, P6, P8;
-                    series_polys(T.series, sr, X.h, P4, P6, P8);
-                    const Pair f = add_small(
-                        {y.h, y.l + (series_value(P4, P6, P8, y.h, y2.h) + series_tenth(T.series, sr, X.h, y.h, y2.h))}, v);
+                    float higher = 0.0f;
+                    if (y.h > kSeriesEnds) {
+                        float P4, P6, P8;
+                        series_polys(T.series, sr, X.h, P4, P6, P8);
+                        higher = series_value(P4, P6, P8, y.h, y2.h) + series_tenth(T.series, sr, X.h, y.h, y2.h);
+                    }
+                    const Pair f = add_small({y.h, y.l + higher}, v);
                     acc[j] += T.vol * ((double)rho * (((double)f.h + (double)f.l) * inv) - (double)(rho * pm));
                 }
             }

@@ -2,7 +2,10 @@
 
 * step cap: the largest integer is no cap at all;
 * double-precision normals: every digit of the small ones too;
+* boundary tables: grids of many cells in a row;
 """
+import os
+
 import numpy as np
 import pytest
 import torch
@@ -12,8 +15,10 @@ from paper_1709_07469_gb300 import build as B
 from paper_1709_07469_gb300 import mcgrav as M
 from paper_1709_07469_gb300 import workloads as W
 from paper_1709_07469_gb300.device import DeviceSolve
+from tests.helpers import oracle_spec
 
 pytestmark = pytest.mark.gpu
+THREADS = os.cpu_count() or 1
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -50,3 +55,49 @@ def test_fp64_normals_keep_their_leading_digits():
     got, want = out.cpu().numpy(), oracle.normals(11, 3, 5, 0, nb)
     assert np.abs(want).min() < 1e-5
     assert np.all(np.abs(got - want) <= 6 * 2.0**-52 * np.abs(want))
+
+
+def box_of_cells(shape, side, air=0.0):
+    """A voxel workload whose domain is its grid of cubes, `air` more above it."""
+    n = np.array(shape, dtype=np.float64) * side
+    w = W.voxel_survey(shape=shape).with_(g_kind="zero", G=1.0)
+    return w.with_(lo=tuple(-0.5 * n), hi=tuple(0.5 * n + np.array([0.0, 0.0, air])), grid_origin=tuple(-0.5 * n),
+                   grid_spacing=(side, side, side))
+
+
+@pytest.mark.parametrize("shape", [(1, 3000, 1), (2, 20000, 1), (1, 200000, 1), (1, 1, 20000)])
+def test_tables_of_long_thin_grids(shape):
+    """A near zone over a grid of up to 2e5 cells in a row.  Reference: direct
+    prism sums of the 64 cells next to the node's end (beyond, they cancel), point
+    masses in doubles for the others (a cube's next term: 0.2 (1 / 128)^4 of its
+    own).  Result rounded to single precision, allowance 3e-7 as in
+    test_gpu_setup.py."""
+    w = box_of_cells(shape, 10.0)
+    axis = int(np.argmax(shape))
+    rng = np.random.default_rng(axis)
+    grid = rng.uniform(100.0, 500.0, shape[::-1]).astype(np.float32)
+    faces = torch.empty((6, 2, 2), dtype=torch.float32, device="cuda")
+    M.mcg_boundary_tables(M.problem(w, grid=torch.from_numpy(grid).cuda()), 2, 2, 1e6, faces)
+    got = faces.cpu().numpy().astype(np.float64)
+    fi, iv, iu = np.meshgrid(np.arange(6), np.arange(2), np.arange(2), indexing="ij")
+    lo, hi = np.array(w.lo), np.array(w.hi)
+    sp = np.array(w.grid_spacing)
+    along = np.arange(shape[axis])
+    to = [1] * 3
+    to[2 - axis] = -1
+    ends = []
+    for first in (along < 64, along >= shape[axis] - 64):
+        near = np.where(first.reshape(to), grid, 0).astype(np.float32)
+        ends.append((oracle.table_nodes(oracle_spec(w, grid=near), fi.ravel(), iu.ravel(), iv.ravel(), 2, 2,
+                                        threads=THREADS), np.where(first.reshape(to), 0.0, grid.astype(np.float64))))
+    c = [(lo[k] + (np.arange(shape[k]) + 0.5) * sp[k]).reshape([-1 if 2 - k == d else 1 for d in range(3)])
+         for k in range(3)]
+    for e, (f, b, a) in enumerate(zip(fi.ravel(), iv.ravel(), iu.ravel())):
+        k = f // 2
+        p, q = [(1, 2), (0, 2), (0, 1)][k]
+        x = np.zeros(3)
+        x[k], x[p], x[q] = (hi if f % 2 else lo)[k], (hi if a else lo)[p], (hi if b else lo)[q]
+        exact, far = ends[0 if x[axis] < 0.0 else 1]
+        r = np.sqrt((c[0] - x[0]) ** 2 + (c[1] - x[1]) ** 2 + (c[2] - x[2]) ** 2)
+        want = exact[e] - w.G * np.prod(sp) * np.sum(far / r)
+        np.testing.assert_allclose(got[f, b, a], want, rtol=3e-7)
