@@ -131,6 +131,7 @@ struct TableParams {
     double vol;              // cell volume
     double near2;            // squared radius of the exact (near) zone
     double unit;             // longest side of a cell
+    double core_least;       // half-width of the core of a small near zone
     double second[3];        // cell_series for lengths in units of `unit`: its order 2 ...
     float series[kSeriesTerms];  // ... and all of it in single precision
     double G;
@@ -140,14 +141,16 @@ struct TableParams {
 constexpr int kTableThreads = 256;
 constexpr int kTableWarps = kTableThreads / 32;
 constexpr int kRowsPerTile = 8;
-// In units of the longest side, along every axis: cells up to kCoreSides from
-// the node are summed by grid node (exact); of the others in the near zone
-// those up to kExactSides as exact prisms (there are some only where the zone
-// is smaller than the core), the rest by the series of mcg_cell.cuh, whose
-// remainder beyond the core is about 1e-11 of the cell's own term: with the
-// core at three sides and without P_10 (1e-8) one table value in a thousand
-// rounded to its neighbour.
-constexpr double kCoreSides = 4.0, kExactSides = 2.0;
+// Cells of the near zone up to kCoreSides of the longest side from the node,
+// along every axis, are summed by grid node (exact), the rest by the series of
+// mcg_cell.cuh, whose remainder is 4e-12 of the cell's own term there: without
+// P_10 (1e-8) one table value in a thousand rounded to its neighbour.  A smaller
+// zone's core is the box inside it, down to core_least: three sides (1e-10), or
+// 2.25 for cells of 1 : 0.6 and longer (at most 9e-10; with three, 128 x 24 x 64
+// cells and a zone of four diagonals took 10.3 ms for 6 x 21^2 nodes instead of
+// 4.9).  Below that the core stays as large and each of its cells is asked
+// whether it is near.
+constexpr double kCoreSides = 4.0, kCoreLeast = 3.0, kCoreLeastLong = 2.25, kLong = 0.6;
 // Beyond 2048 sides P_4 .. P_10 add less than 1e-15 of the cell's term (0.015 y^4,
 // below the pairs' 3e-14), and powers of coordinates counted in sides overflow
 // from 1.6e4 sides on (inf times an underflown y^20 is no number).
@@ -165,6 +168,14 @@ __device__ __forceinline__ void node_position(const TableParams& T, int64_t node
     x[a] = T.lo[a] + (T.hi[a] - T.lo[a]) * (double)iu / (double)(T.nu - 1);
     x[b] = T.lo[b] + (T.hi[b] - T.lo[b]) * (double)iv / (double)(T.nv - 1);
 }
+
+// Offset of a cell's centre along an axis, and the squared distance (rounded
+// alike wherever a cell is asked whether it is near).
+__device__ __forceinline__ double cell_offset(const TableParams& T, int k, int i, double x)
+{
+    return __dadd_rn(__fma_rn((double)i + 0.5, T.sp[k], T.org[k]), -x);
+}
+__device__ __forceinline__ double square_sum(double a, double b2) { return __fma_rn(a, a, b2); }
 
 // Point-mass far field for every voxel (single-precision terms, summed per
 // row in single precision and per row into double), then, for voxels whose
@@ -265,8 +276,10 @@ __global__ void __launch_bounds__(kTableThreads, 2) tables_kernel(const TablePar
             ihi[k] = (int)b;
         }
         if (ilo[0] > ihi[0] || ilo[1] > ihi[1] || ilo[2] > ihi[2]) continue;
-        // the core: a box of cells inside the near zone
-        const double core = fmin(kCoreSides * T.unit, R * 0.57);
+        // the core: a box of cells inside the near zone (its half-width is below
+        // R / sqrt 3), or of cells to be asked
+        const bool whole = R * 0.57 >= T.core_least;
+        const double core = whole ? fmin(kCoreSides * T.unit, R * 0.57) : fmin(T.core_least, R);
         int clo[3], chi[3];
         for (int k = 0; k < 3; ++k) {
             const double a = (x[k] - T.org[k]) / T.sp[k], w = core / T.sp[k];
@@ -276,18 +289,17 @@ __global__ void __launch_bounds__(kTableThreads, 2) tables_kernel(const TablePar
         const int wy = ihi[1] - ilo[1] + 1, box_rows = wy * (ihi[2] - ilo[2] + 1);
         for (int q = part * kTableWarps + warp; q < box_rows; q += kTableWarps * parts) {
             const int iy = ilo[1] + q % wy, iz = ilo[2] + q / wy;
-            const double cy = T.org[1] + (iy + 0.5) * T.sp[1] - x[1], cz = T.org[2] + (iz + 0.5) * T.sp[2] - x[2];
-            const double cyz = cy * cy + cz * cz;
+            const double cy = cell_offset(T, 1, iy, x[1]), cz = cell_offset(T, 2, iz, x[2]);
+            const double cyz = square_sum(cy, __dmul_rn(cz, cz));
             if (cyz >= T.near2) continue;
             const bool core_row = iy >= clo[1] && iy < chi[1] && iz >= clo[2] && iz < chi[2];
-            const bool exact_row = fabs(cy) < kExactSides * T.unit && fabs(cz) < kExactSides * T.unit;
             const double Y = cy * cy * inv2, Z = cz * cz * inv2;
             const SeriesRow sr = series_row(T.series, (float)Y, (float)Z);
             const Pair p2x = pair_of(T.second[0]), c2 = pair_of(T.second[1] * Y + T.second[2] * Z);
             const float dy = (float)iy * sy - py[j], dz = (float)iz * sz - pz[j];
             for (int ix = ilo[0]; ix <= ihi[0]; ++ix) {
-                const double cx = T.org[0] + (ix + 0.5) * T.sp[0] - x[0];
-                const double d2 = cx * cx + cyz;
+                const double cx = cell_offset(T, 0, ix, x[0]);
+                const double d2 = square_sum(cx, cyz);
                 if (d2 >= T.near2) continue;
                 const float rho = __ldg(T.grid + ((int64_t)iz * T.ny + iy) * T.nx + ix);
                 if (rho == 0.0f) continue;
@@ -296,12 +308,6 @@ __global__ void __launch_bounds__(kTableThreads, 2) tables_kernel(const TablePar
                 asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(pm) : "f"(fmaf(dx, dx, fmaf(dy, dy, dz * dz))));
                 if (core_row && ix >= clo[0] && ix < chi[0]) {
                     acc[j] -= T.vol * (double)(rho * pm);  // its own potential: the core's node sum
-                } else if (exact_row && fabs(cx) < kExactSides * T.unit) {
-                    const double lo[3] = {T.org[0] + ix * T.sp[0], T.org[1] + iy * T.sp[1], T.org[2] + iz * T.sp[2]};
-                    const double hi[3] = {lo[0] + T.sp[0], lo[1] + T.sp[1], lo[2] + T.sp[2]};
-                    // (returns -G rho [[[F]]]; with G = -1 it gives +rho [[[F]]])
-                    const double exact = prism_potential_paired(-1.0, (double)rho, lo, hi, x);
-                    acc[j] += exact - T.vol * (double)(rho * pm);
                 } else {
                     const Pair X = pair_of(cx * cx * inv2);
                     Pair y2, P2, y5;
@@ -330,8 +336,13 @@ __global__ void __launch_bounds__(kTableThreads, 2) tables_kernel(const TablePar
             for (int m = 0; m < 8; ++m) {
                 const int ci = a - 1 + (m & 1), cj = b - 1 + ((m >> 1) & 1), ck = c - 1 + (m >> 2);
                 double v = 0.0;
-                if (ci >= clo[0] && ci < chi[0] && cj >= clo[1] && cj < chi[1] && ck >= clo[2] && ck < chi[2])
-                    v = (double)__ldg(T.grid + ((int64_t)ck * T.ny + cj) * T.nx + ci);
+                bool in = ci >= clo[0] && ci < chi[0] && cj >= clo[1] && cj < chi[1] && ck >= clo[2] && ck < chi[2];
+                if (!whole) {
+                    const double cz = cell_offset(T, 2, ck, x[2]);
+                    const double cyz = square_sum(cell_offset(T, 1, cj, x[1]), __dmul_rn(cz, cz));
+                    in = in && square_sum(cell_offset(T, 0, ci, x[0]), cyz) < T.near2;
+                }
+                if (in) v = (double)__ldg(T.grid + ((int64_t)ck * T.ny + cj) * T.nx + ci);
                 w += ((m ^ (m >> 1) ^ (m >> 2)) & 1) ? -v : v;
             }
             if (w != 0.0)
@@ -492,6 +503,8 @@ int boundary_tables(const mcg_domain* d, const mcg_density* rho, int32_t nu, int
     T.out = faces_out;
     const int64_t nodes = 6ll * nu * nv;
     T.unit = std::max(T.sp[0], std::max(T.sp[1], T.sp[2]));
+    const double second = T.sp[0] + T.sp[1] + T.sp[2] - T.unit - std::min(T.sp[0], std::min(T.sp[1], T.sp[2]));
+    T.core_least = (second > kLong * T.unit ? kCoreLeast : kCoreLeastLong) * T.unit;
     const double half[3] = {0.5 * T.sp[0] / T.unit, 0.5 * T.sp[1] / T.unit, 0.5 * T.sp[2] / T.unit};
     double series[kSeriesTerms];
     cell_series(half, series);

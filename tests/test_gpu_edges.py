@@ -2,7 +2,7 @@
 
 * step cap: the largest integer is no cap at all;
 * double-precision normals: every digit of the small ones too;
-* boundary tables: grids of many cells in a row;
+* boundary tables: grids of many cells in a row; near zones of a few cells;
 """
 import os
 
@@ -101,3 +101,20 @@ def test_tables_of_long_thin_grids(shape):
         r = np.sqrt((c[0] - x[0]) ** 2 + (c[1] - x[1]) ** 2 + (c[2] - x[2]) ** 2)
         want = exact[e] - w.G * np.prod(sp) * np.sum(far / r)
         np.testing.assert_allclose(got[f, b, a], want, rtol=3e-7)
+
+
+@pytest.mark.parametrize("near", [1.5, 2.0, 3.0])
+def test_tables_of_a_cell_at_the_rim_of_a_small_near_zone(near):
+    """A dense cell two to four of its sides below a node: its own prism potential,
+    rounded to single precision (half a unit in the last place; the sums before
+    are doubles: 1e-3 of one more)."""
+    w = box_of_cells((1, 1, 1), 1.0)
+    grid = torch.full((1, 1, 1), 500.0, dtype=torch.float32, device="cuda")
+    faces = torch.empty((6, 3, 3), dtype=torch.float32, device="cuda")
+    gaps = np.linspace(1.5, min(near * np.sqrt(3.0), 4.2) - 0.51, 200)
+    for gap in gaps:
+        v = w.with_(hi=(0.5, 0.5, 0.5 + gap))
+        M.mcg_boundary_tables(M.problem(v, grid=grid), 3, 3, near, faces)
+        got = faces[5, 1, 1].item()
+        want = oracle.prism_phi(1.0, 500.0, (-0.5, -0.5, -0.5), (0.5, 0.5, 0.5), (0.0, 0.0, 0.5 + gap))
+        assert abs(got - want) <= 0.501 * np.spacing(np.float32(abs(want))), gap
