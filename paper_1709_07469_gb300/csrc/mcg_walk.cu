@@ -155,7 +155,7 @@ template <int RHO>
 __device__ __forceinline__ double recorded_sum(const WalkParams& P, unsigned long long acc)
 {
     if constexpr (kTwoValued<RHO>)
-        return (double)P.rho0_f * (0.5 * (double)(long long)acc);
+        return acc ? (double)P.rho0_f * (0.5 * (double)(long long)acc) : 0.0;  // (0 for any rho0)
     else
         return __longlong_as_double((long long)acc);
 }

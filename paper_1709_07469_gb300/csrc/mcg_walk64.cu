@@ -603,7 +603,8 @@ __global__ void __launch_bounds__(128, 4) walk64_kernel(const WalkParams P, cons
                         // (the moves' place holds positions now)
                         step_of(tables, P.sd, make_uint4(3u * myblk, gp, gs, 0u), gk0, gk1, m, e.dW);
                         e.face = (int)((of >> (3 * c)) & 7u) - 1;
-                        if constexpr (kTwoValued<RHO>) e.sum = 0.5 * P.rho0 * (double)(long long)w.acc[c];
+                        if constexpr (kTwoValued<RHO>)  // (0 for any rho0 where the walk never met the body)
+                            e.sum = w.acc[c] ? 0.5 * P.rho0 * (double)(long long)w.acc[c] : 0.0;
                         else e.sum = __longlong_as_double((long long)w.acc[c]);
                         atomicAdd(&w.steps, (unsigned long long)nstep_of(myblk, m));
                     }

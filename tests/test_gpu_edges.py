@@ -2,6 +2,7 @@
 
 * step cap: the largest integer is no cap at all;
 * double-precision normals: every digit of the small ones too;
+* a density that is not finite: only the walks that meet it;
 * boundary tables: grids of many cells in a row; near zones of a few cells;
 """
 import os
@@ -118,3 +119,28 @@ def test_tables_of_a_cell_at_the_rim_of_a_small_near_zone(near):
         got = faces[5, 1, 1].item()
         want = oracle.prism_phi(1.0, 500.0, (-0.5, -0.5, -0.5), (0.5, 0.5, 0.5), (0.0, 0.0, 0.5 + gap))
         assert abs(got - want) <= 0.501 * np.spacing(np.float32(abs(want))), gap
+
+
+@pytest.mark.parametrize("precision", [M.MCG_FP64, M.MCG_MIXED])
+@pytest.mark.parametrize("rho0", [float("inf"), float("nan")])
+@pytest.mark.parametrize("kind", ["prism", "sphere"])
+def test_nonfinite_density_reaches_only_the_walks_that_meet_it(precision, rho0, kind):
+    """With zero boundary data a walk that never met the body has u = 0 for any
+    density of the body; only the others are lost to a density that is not finite."""
+    w = W.prism_ore_body(paths=512, step=20.0) if kind == "prism" else W.sphere_line(paths=512)
+    st = w.stations[:1] if kind == "prism" else np.array([[0.0, 0.0, 0.9]])
+    w = w.with_(g_kind="zero", stations=st)
+    met = None
+    for r in (w.rho0, rho0):
+        ds = DeviceSolve(w.with_(rho0=r), precision=precision)
+        ds.reset()
+        ds.walk(0)
+        u = ds.per_path()[0]
+        status = int(ds.status[0].item())
+        if met is None:
+            met = u != 0.0
+            assert 0 < met.sum() < met.size and status == 0
+        else:
+            assert np.all(u[~met] == 0.0)
+            assert not np.any(np.isfinite(u[met]))
+            assert status == 1 << M.MCG_ERR_NONFINITE
