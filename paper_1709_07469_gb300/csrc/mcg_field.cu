@@ -477,9 +477,9 @@ extern "C" int mcg_field(const mcg_density* density, const double* points_dev, i
         cfg.attrs = &at;
         cfg.numAttrs = 1;
         const bool cube = P.series[0] == 0.0 && P.series[1] == 0.0 && P.series[2] == 0.0;
-        const cudaError_t le = cube ? cudaLaunchKernelEx(&cfg, field_voxel_kernel<true>, P)
-                                    : cudaLaunchKernelEx(&cfg, field_voxel_kernel<false>, P);
-        if (le != cudaSuccess) return set_error(MCG_ERR_CUDA, "field kernel launch: %s", cudaGetErrorString(le));
+        // (its error, if any, is read and cleared below)
+        if (cube) cudaLaunchKernelEx(&cfg, field_voxel_kernel<true>, P);
+        else cudaLaunchKernelEx(&cfg, field_voxel_kernel<false>, P);
         break;
     }
     default:

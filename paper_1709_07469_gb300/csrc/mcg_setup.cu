@@ -528,8 +528,9 @@ int boundary_tables(const mcg_domain* d, const mcg_density* rho, int32_t nu, int
     at.val.clusterDim.y = at.val.clusterDim.z = 1;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    const cudaError_t e = many ? cudaLaunchKernelEx(&cfg, tables_kernel<2>, T)
-                               : cudaLaunchKernelEx(&cfg, tables_kernel<1>, T);
+    if (many) cudaLaunchKernelEx(&cfg, tables_kernel<2>, T);
+    else cudaLaunchKernelEx(&cfg, tables_kernel<1>, T);
+    const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? MCG_OK : set_error(MCG_ERR_CUDA, "tables kernel: %s", cudaGetErrorString(e));
 }
 

@@ -694,8 +694,9 @@ cudaError_t launch_walk64(const WalkParams& P0, int block, int blocks, cudaStrea
     const int grid = need < (long long)blocks ? (int)need : blocks;
     Near T = make_near(P);
     void* args[2] = {&P, &T};
-    return cudaLaunchKernel(walk64_fn(P.rho_kind, P.crn != 0, P.seg != nullptr), dim3((unsigned)(grid > 0 ? grid : 1)),
-                            dim3((unsigned)block), args, 0, st);
+    cudaLaunchKernel(walk64_fn(P.rho_kind, P.crn != 0, P.seg != nullptr), dim3((unsigned)(grid > 0 ? grid : 1)),
+                     dim3((unsigned)block), args, 0, st);
+    return cudaGetLastError();
 }
 
 void preload_walk64_kernels()

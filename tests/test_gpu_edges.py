@@ -4,7 +4,9 @@
 * double-precision normals: every digit of the small ones too;
 * a density that is not finite: only the walks that meet it;
 * boundary tables: grids of many cells in a row; near zones of a few cells;
+* an error of one launch is not reported by the next;
 """
+import ctypes
 import os
 
 import numpy as np
@@ -144,3 +146,47 @@ def test_nonfinite_density_reaches_only_the_walks_that_meet_it(precision, rho0, 
             assert np.all(u[~met] == 0.0)
             assert not np.any(np.isfinite(u[met]))
             assert status == 1 << M.MCG_ERR_NONFINITE
+
+
+def invalid_stream():
+    """A stream whose capture has been broken: whatever is launched into it is
+    refused.  Returns (stream, end): nothing is left of it after end()."""
+    cu = ctypes.CDLL("libcuda.so.1")
+    st = ctypes.c_void_p()
+    assert cu.cuStreamCreate(ctypes.byref(st), 1) == 0
+    assert cu.cuStreamBeginCapture_v2(st, 2) == 0          # (relaxed: other streams are not concerned)
+    assert cu.cuStreamSynchronize(st) != 0                 # not allowed in a capture: ends it with an error
+
+    def end():
+        graph = ctypes.c_void_p()
+        assert cu.cuStreamEndCapture(st, ctypes.byref(graph)) != 0
+        assert cu.cuStreamDestroy_v2(st) == 0
+
+    return st.value, end
+
+
+@pytest.mark.parametrize("call", ["field", "tables"])
+def test_a_refused_launch_leaves_no_error_behind(call):
+    w, grid = box_of_cells((4, 4, 4), 1.0), torch.ones((4, 4, 4), dtype=torch.float32, device="cuda")
+    prob = M.problem(w, grid=grid)
+    x = torch.full((1, 3), 5.0, dtype=torch.float64, device="cuda")
+    phi = torch.empty(1, dtype=torch.float64, device="cuda")
+    faces = torch.empty((6, 2, 2), dtype=torch.float32, device="cuda")
+
+    def field(stream):
+        M.mcg_field(prob, x, 1, phi, None, stream)
+
+    def tables(stream):
+        M.mcg_boundary_tables(prob, 2, 2, 4.0, faces, stream)
+
+    torch.cuda.synchronize()
+    st, end = invalid_stream()
+    try:
+        with pytest.raises(M.McgError):
+            (field if call == "field" else tables)(st)
+    finally:
+        end()
+    for good in (tables, field):
+        good(None)
+    torch.cuda.synchronize()
+    assert np.isfinite(phi.item()) and np.all(np.isfinite(faces.cpu().numpy()))
