@@ -54,8 +54,8 @@ bool host_memory(const void* p)
 
 // mcgrav_solve's workspaces come from a stream-ordered pool of the library's
 // own, one per device: a cudaMalloc and cudaFree pair took most of the 230 us
-// of a smallest solve (78 us now).  The pool hands memory back to the device beyond
-// kPoolKeeps, and serves any number of threads and streams.
+// of a smallest solve (78 us now).  The pool keeps kPoolKeeps for later calls, and
+// serves any number of threads and streams.
 constexpr uint64_t kPoolKeeps = 256ull << 20;
 
 cudaError_t solve_pool(cudaMemPool_t* pool)
@@ -85,6 +85,18 @@ cudaError_t solve_pool(cudaMemPool_t* pool)
     }
     *pool = pools[dev];
     return cudaSuccess;
+}
+
+// Ends the use of a workspace (in stream order).  The pool acts on its threshold
+// only when something synchronises later, so what it holds beyond it is handed
+// back here; the wait is for the release alone, the caller has waited for the rest.
+void release_workspace(cudaMemPool_t pool, void* ws, cudaStream_t st)
+{
+    cudaFreeAsync(ws, st);
+    uint64_t held = 0;
+    if (cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &held) == cudaSuccess && held > kPoolKeeps &&
+        cudaStreamSynchronize(st) == cudaSuccess)
+        cudaMemPoolTrimTo(pool, kPoolKeeps);
 }
 
 // mcgrav_solve's workspace: a shared part (stations, finalized results, status
@@ -636,7 +648,7 @@ int mcgrav_solve(const mcg_domain* domain, const mcg_density* density, const mcg
 
     double* h_res = new (std::nothrow) double[res_bytes / sizeof(double) + 1];
     if (!h_res) {
-        cudaFreeAsync(ws, st);
+        release_workspace(pool, ws, st);
         return set_error(MCG_ERR_OOM, "host results of %lld stations", (long long)S);
     }
     int32_t h_status = 0;
@@ -757,9 +769,10 @@ int mcgrav_solve(const mcg_domain* domain, const mcg_density* density, const mcg
         }
         rc = status_from_bits(h_status);
     } while (0);
-    if (rc == MCG_ERR_CUDA) cudaStreamSynchronize(st);
+    // after an error, whatever has been queued may still read the caller's arrays
+    if (rc) cudaStreamSynchronize(st);
     delete[] h_res;
-    cudaFreeAsync(ws, st);  // (nothing queued uses it any more)
+    release_workspace(pool, ws, st);
     return rc;
 }
 

@@ -5,6 +5,7 @@
 * a density that is not finite: only the walks that meet it;
 * boundary tables: grids of many cells in a row; near zones of a few cells;
 * an error of one launch is not reported by the next;
+* mcgrav_solve: its workspace goes back, and a failed call waits as well;
 """
 import ctypes
 import os
@@ -190,3 +191,35 @@ def test_a_refused_launch_leaves_no_error_behind(call):
         good(None)
     torch.cuda.synchronize()
     assert np.isfinite(phi.item()) and np.all(np.isfinite(faces.cpu().numpy()))
+
+
+def used_bytes():
+    free, total = torch.cuda.mem_get_info()
+    return total - free
+
+
+def test_solve_hands_its_workspace_back():
+    """At most 256 MiB of a solve's workspace stay with the library after the
+    call, without a further synchronisation."""
+    w = W.sphere_line(dt=0.04)
+    opts = M.options(w, batch_paths=1 << 18)
+    M.mcgrav_solve(M.problem(w), w.stations, 64, w.dt, 0, M.options(w))
+    torch.cuda.synchronize()
+    before = used_bytes()
+    assert M.mcg_workspace_bytes(8, 1 << 18) > (512 << 20)
+    M.mcgrav_solve(M.problem(w), w.stations, 1 << 19, w.dt, 0, opts)
+    assert used_bytes() - before <= 256 << 20
+
+
+def test_a_failed_solve_waits_for_its_copies():
+    """A grid of one layer too large to pack is refused after its copy to the
+    device has been queued: the call returns once the copy is done, as the
+    caller's (pinned) array may go away then."""
+    nx, ny = 1 << 15, (1 << 31) // 3 // (1 << 15) + 1
+    w = box_of_cells((8, 8, 8), 10.0).with_(g_kind="zero", stations=np.zeros((1, 3)), paths=1)
+    grid = torch.empty((1, ny, nx), dtype=torch.float32, pin_memory=True)
+    prob = M.problem(w, grid=grid.numpy())
+    st = torch.cuda.Stream()
+    r = M.mcgrav_solve(prob, w.stations, 1, w.dt, 0, M.options(w, stream=st), allow=(M.MCG_ERR_ARG,))
+    assert st.query()
+    assert r.status == M.MCG_ERR_ARG and "too large to pack" in M.last_error()
