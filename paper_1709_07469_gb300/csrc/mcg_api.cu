@@ -9,7 +9,9 @@
 #include <atomic>
 #include <mutex>
 #include <new>
+#include <vector>
 
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include "mcg_internal.h"
@@ -52,38 +54,64 @@ bool host_memory(const void* p)
     return a.type == cudaMemoryTypeUnregistered || a.type == cudaMemoryTypeHost;
 }
 
+// Identity of the current context, which no other has in the process: a device
+// reset ends the context, and a pool made in it is not to be touched again.
+cudaError_t context_id(unsigned long long* id)
+{
+    using Fn = CUresult (*)(CUcontext, unsigned long long*);
+    static const Fn fn = [] {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        const cudaError_t e = cudaGetDriverEntryPointByVersion("cuCtxGetId", &p, 12000, cudaEnableDefault, &found);
+        return e == cudaSuccess && found == cudaDriverEntryPointSuccess ? (Fn)p : (Fn) nullptr;
+    }();
+    if (!fn) return cudaErrorNotSupported;
+    if (fn(nullptr, id) == CUDA_SUCCESS) return cudaSuccess;
+    const cudaError_t e = cudaFree(nullptr);  // (no context yet: the device's own becomes current)
+    if (e != cudaSuccess) return e;
+    return fn(nullptr, id) == CUDA_SUCCESS ? cudaSuccess : cudaErrorDeviceUninitialized;
+}
+
 // mcgrav_solve's workspaces come from a stream-ordered pool of the library's
-// own, one per device: a cudaMalloc and cudaFree pair took most of the 230 us
+// own, one per context: a cudaMalloc and cudaFree pair took most of the 230 us
 // of a smallest solve (78 us now).  The pool keeps kPoolKeeps for later calls, and
 // serves any number of threads and streams.
 constexpr uint64_t kPoolKeeps = 256ull << 20;
 
 cudaError_t solve_pool(cudaMemPool_t* pool)
 {
+    struct Entry {
+        unsigned long long context;
+        cudaMemPool_t pool;
+    };
     static std::mutex mu;
-    static cudaMemPool_t pools[64] = {};
+    static std::vector<Entry> pools;
+    unsigned long long id = 0;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = context_id(&id);
     if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     std::lock_guard<std::mutex> lk(mu);
-    if (!pools[dev]) {
-        cudaMemPoolProps props;
-        std::memset(&props, 0, sizeof(props));
-        props.allocType = cudaMemAllocationTypePinned;
-        props.handleTypes = cudaMemHandleTypeNone;
-        props.location.type = cudaMemLocationTypeDevice;
-        props.location.id = dev;
-        cudaMemPool_t p = nullptr;
-        if ((e = cudaMemPoolCreate(&p, &props))) return e;
-        uint64_t keep = kPoolKeeps;
-        if ((e = cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep))) {
-            cudaMemPoolDestroy(p);
-            return e;
+    for (const Entry& p : pools)
+        if (p.context == id) {
+            *pool = p.pool;
+            return cudaSuccess;
         }
-        pools[dev] = p;
+    cudaMemPoolProps props;
+    std::memset(&props, 0, sizeof(props));
+    props.allocType = cudaMemAllocationTypePinned;
+    props.handleTypes = cudaMemHandleTypeNone;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t p = nullptr;
+    if ((e = cudaMemPoolCreate(&p, &props))) return e;
+    uint64_t keep = kPoolKeeps;
+    if ((e = cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep))) {
+        cudaMemPoolDestroy(p);
+        return e;
     }
-    *pool = pools[dev];
+    pools.push_back({id, p});
+    *pool = p;
     return cudaSuccess;
 }
 

@@ -6,9 +6,12 @@
 * boundary tables: grids of many cells in a row; near zones of a few cells;
 * an error of one launch is not reported by the next;
 * mcgrav_solve: its workspace goes back, and a failed call waits as well;
+* mcgrav_solve after a device reset;
 """
 import ctypes
 import os
+import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -223,3 +226,39 @@ def test_a_failed_solve_waits_for_its_copies():
     r = M.mcgrav_solve(prob, w.stations, 1, w.dt, 0, M.options(w, stream=st), allow=(M.MCG_ERR_ARG,))
     assert st.query()
     assert r.status == M.MCG_ERR_ARG and "too large to pack" in M.last_error()
+
+
+RESET = """
+import ctypes, os
+import numpy as np
+from paper_1709_07469_gb300 import mcgrav as M, workloads as W
+
+M.load()
+w = W.sphere_line(dt=0.01)
+
+
+def solve():
+    return M.mcgrav_solve(M.problem(w), w.stations, 64, w.dt, 0, M.options(w)).u
+
+
+first = solve()
+for _ in range(3):
+    assert ctypes.CDLL(os.environ["CUDART"]).cudaDeviceReset() == 0
+    for _ in range(2):
+        assert np.array_equal(solve(), first)
+"""
+
+
+def cudart():
+    with open("/proc/self/maps") as f:
+        found = {line.split()[-1] for line in f if "libcudart.so" in line}
+    return found.pop()
+
+
+def test_solve_after_a_device_reset():
+    """The program's own runtime resets the device (its process alone is
+    concerned): the library takes up a new context."""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", RESET], cwd=root, env=dict(os.environ, CUDART=cudart(), PYTHONPATH=root),
+                       capture_output=True, text=True, timeout=120)
+    assert r.returncode == 0, r.stderr
