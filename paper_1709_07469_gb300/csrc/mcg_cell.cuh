@@ -8,9 +8,11 @@
 //
 // the Taylor series of 1 / r averaged term by term.  P_2n is a homogeneous
 // harmonic polynomial of degree 2n in the squares X, Y, Z of d's coordinates.
-// Kept up to n = 4 (the field) or 5 (the tables): the relative remainder of
-// n <= 4 for a cube is 4e-10 at four sides and 7e-12 at six (compared with
-// 14^3-point Gauss quadrature for four cell shapes, the cube the worst).
+// Kept up to n = 4 (the field; n = 5 next to its near zone) or 5 (the tables):
+// the relative remainder of n <= 4 for a cube is 4e-10 at four sides and 7e-12 at
+// six (compared with 14^3-point Gauss quadrature for four cell shapes, the cube
+// the worst); that of n <= 5 is 1e-8 at two sides, 1e-10 at three, 4e-12 at four
+// (against the closed form in 40 digits).
 // Along a row of cells (Y, Z fixed) every P_2n is a short polynomial in X.
 #pragma once
 #include <cuda_runtime.h>
@@ -44,6 +46,12 @@ __device__ __forceinline__ Pair add(Pair a, Pair b)
     const float h = __fadd_rn(a.h, b.h), t = __fsub_rn(h, a.h);
     const float e = __fadd_rn(__fsub_rn(a.h, __fsub_rn(h, t)), __fsub_rn(b.h, t));
     return {h, e + (a.l + b.l)};
+}
+// The same number, its leading part the nearest float.
+__device__ __forceinline__ Pair rounded(Pair a)
+{
+    const float h = __fadd_rn(a.h, a.l);
+    return {h, __fsub_rn(a.l, __fsub_rn(h, a.h))};
 }
 // a + b, |a| >= |b|
 __device__ __forceinline__ Pair add_small(Pair a, Pair b)
@@ -114,17 +122,22 @@ __device__ __forceinline__ float series_tenth(const float* p, const SeriesRow& r
     return y8 * y8 * y4 * y * P10;
 }
 
-// The same terms (n = 2, 3, 4) of (df/dz) / d_z: 2 dP_2n/dZ y^(4n+1) - (4n+1) P_2n y^(4n+3).
+// The same terms (n = 2, 3, 4) of (df/dz) / d_z: 2 dP_2n/dZ y^(4n+1) - (4n+1) P_2n y^(4n+3);
+// n = 3 and 4 by y^13.
+__device__ __forceinline__ float slope_rest(const float* p, const SeriesRow& r, float X, float P6, float P8, float y2)
+{
+    const float D6 = fmaf(fmaf(p[11], X, r.d6[0]), X, r.d6[1]);
+    const float D8 = fmaf(fmaf(fmaf(p[21], X, r.d8[0]), X, r.d8[1]), X, r.d8[2]);
+    const float t6 = fmaf(-13.0f * y2, P6, 2.0f * D6), t8 = fmaf(-17.0f * y2, P8, 2.0f * D8);
+    return fmaf(y2 * y2, t8, t6);
+}
 __device__ __forceinline__ float series_slope(const float* p, const SeriesRow& r, float X, float P4, float P6,
                                               float P8, float y, float y2)
 {
     const float D4 = fmaf(p[5], X, r.d4);
-    const float D6 = fmaf(fmaf(p[11], X, r.d6[0]), X, r.d6[1]);
-    const float D8 = fmaf(fmaf(fmaf(p[21], X, r.d8[0]), X, r.d8[1]), X, r.d8[2]);
-    const float t4 = fmaf(-9.0f * y2, P4, 2.0f * D4), t6 = fmaf(-13.0f * y2, P6, 2.0f * D6),
-                t8 = fmaf(-17.0f * y2, P8, 2.0f * D8);
+    const float t4 = fmaf(-9.0f * y2, P4, 2.0f * D4);
     const float y4 = y2 * y2;
-    return y4 * y4 * y * fmaf(y4, fmaf(y4, t8, t6), t4);
+    return y4 * y4 * y * fmaf(y4, slope_rest(p, r, X, P6, P8, y2), t4);
 }
 
 // P_2 y^5, the second-order term of a cell that is not a cube (P_2 = 0 for
@@ -153,6 +166,38 @@ __device__ __forceinline__ Pair rsqrt_pair(Pair s, Pair& y2)
     y.l = y.h * e * fmaf(0.375f, e, 0.5f);
     y2.l = fmaf(2.0f * y.h, y.l, y2.l);
     return y;
+}
+
+// What series_value and series_slope lack of a cell's own terms, in single
+// precision: the digits of P_4's (as pairs; p4: its coefficients), and P_10's.
+__device__ __forceinline__ void series_lacks(const float* p, const Pair* p4, Pair X, Pair Y, Pair Z, float& f, float& g)
+{
+    const SeriesRow r = series_row(p, Y.h, Z.h);
+    Pair y2;
+    const Pair y = rsqrt_pair(add(X, rounded(add(Y, Z))), y2);
+    float P4, P6, P8;
+    series_polys(p, r, X.h, P4, P6, P8);
+    const float v = series_value(P4, P6, P8, y.h, y2.h), s = series_slope(p, r, X.h, P4, P6, P8, y.h, y2.h);
+    const float y4 = y2.h * y2.h, y13 = y4 * y4 * y4 * y.h;
+    const float v68 = y13 * fmaf(y4, P8, P6), s68 = y13 * slope_rest(p, r, X.h, P6, P8, y2.h);
+    // P_10
+    const float *q = p + 34, Zd = Z.h * Z.h, Zt = Zd * Z.h;
+    const float d3 = fmaf(q[4], Y.h, 2.0f * q[5] * Z.h);
+    const float d2 = fmaf(fmaf(q[7], Y.h, 2.0f * q[8] * Z.h), Y.h, 3.0f * q[9] * Zd);
+    const float d1 = fmaf(fmaf(fmaf(q[11], Y.h, 2.0f * q[12] * Z.h), Y.h, 3.0f * q[13] * Zd), Y.h, 4.0f * q[14] * Zt);
+    const float d0 = fmaf(fmaf(fmaf(fmaf(q[16], Y.h, 2.0f * q[17] * Z.h), Y.h, 3.0f * q[18] * Zd), Y.h,
+                               4.0f * q[19] * Zt), Y.h, 5.0f * q[20] * Zd * Zd);
+    const float D10 = fmaf(fmaf(fmaf(fmaf(q[2], X.h, d3), X.h, d2), X.h, d1), X.h, d0);
+    const float v10 = series_tenth(p, r, X.h, y.h, y2.h), s10 = fmaf(2.0f * D10, y13 * y4 * y4, -21.0f * y2.h * v10);
+    // P_4 and 2 dP_4/dZ - 9 P_4 y^2
+    const Pair a = add(mul(p4[1], Y), mul(p4[2], Z));
+    const Pair b = add(mul(add(mul(p4[3], Y), mul(p4[4], Z)), Y), mul(mul(p4[5], Z), Z));
+    const Pair P = add(mul(add(mul(p4[0], X), a), X), b);
+    const Pair D = add(add(mul(p4[2], X), mul(p4[4], Y)), mul({2.0f, 0.0f}, mul(p4[5], Z)));
+    const Pair u4 = mul(y2, y2), u9 = mul(mul(u4, u4), y);
+    const Pair V = mul(P, u9), S = mul(add(mul({2.0f, 0.0f}, D), mul({-9.0f, 0.0f}, mul(P, y2))), u9);
+    f = ((V.h - v) + v68) + (V.l + v10);
+    g = ((S.h - s) + s68) + (S.l + s10);
 }
 
 // sum += v without losing the rounding of the leading parts.

@@ -29,8 +29,6 @@ namespace mcg {
 
 namespace {
 
-constexpr int kFieldTerms = 3 + 6 + 10 + 15;
-
 struct FieldParams {
     int32_t kind;
     double G, rho0;
@@ -39,7 +37,7 @@ struct FieldParams {
     const float* grid;        // voxel grid, x fastest
     int32_t nx, ny, nz;
     double org[3], sp[3];
-    double series[kFieldTerms];  // cell_series of a cell, up to P_8
+    double series[kSeriesTerms];  // cell_series of a cell
     double near;              // cells with a centre within this of the point (per axis) are summed by node
     const double* x;          // points, n x 3
     int64_t n;
@@ -128,14 +126,50 @@ __global__ void field_closed_kernel(const FieldParams P)
 // 256 points).  Only the cells within kNearCells sides of the point need it;
 // the others take ~95 single-precision instructions: a thread runs a row of
 // cells (its Y, Z polynomials in registers), 16 columns of 256 rows at a time
-// through shared memory so that the grid is read in whole sectors.  Now
-// 2.5 ms (one point 0.29 ms; flat 16 x 128 x 64 cells 9.6 ms).  Error
-// against the 64-bit sum over all nodes: 0.6-2.8e-13 of the field as before,
-// which is that sum's own cancellation.
+// through shared memory so that the grid is read in whole sectors.  What the
+// single-precision terms of the far cells next to the near ones lack (P_4's
+// digits, P_10) is added for them apart, in pairs.  Now 2.6 ms (one point
+// 0.30 ms; flat 16 x 128 x 64 cells 9.6 ms).  Error, in units of the cells' own
+// terms added up, against 64-bit mantissas (nine grids, points on, in and
+// around them): 1e-13 at most, for df/dz (all nodes in doubles: 3e-12; without
+// the rim: 5e-13).
 // ---------------------------------------------------------------------------
 constexpr int kFieldThreads = 256;
 constexpr int kFieldCols = 16;
-constexpr double kNearCells = 6.0;
+constexpr double kNearCells = 6.0, kRimCells = 8.0;
+
+// The rim: far cells up to kRimCells sides from the point, next to the near ones, and
+// what their single-precision terms lack: beyond, 1e-12 of a cell's df/dz.  (A
+// call, and its set-up after the loop over all cells: that loop lost 4 to 6 %
+// with either in its way.)
+struct Rim {
+    int first[3], count[3];  // cells along each axis, the near ones lo .. hi - 1 among them
+    int lo[3], hi[3];
+    Pair d0[3], step[3];     // the first cell's centre, and from cell to cell
+};
+__device__ __noinline__ float2 rim_sum(const float* grid, int nx, int ny, const Rim& R, const float* sp, const Pair* sp4,
+                                       int64_t from, int stride)
+{
+    const int64_t cells = (int64_t)R.count[0] * R.count[1] * R.count[2];
+    float2 sum = {0.0f, 0.0f};
+    for (int64_t q = from; q < cells; q += stride) {
+        const int64_t row = q / R.count[0];
+        const int c[3] = {(int)(q - row * R.count[0]), (int)(row % R.count[1]), (int)(row / R.count[1])};
+        const int ix = R.first[0] + c[0], iy = R.first[1] + c[1], iz = R.first[2] + c[2];
+        if (ix >= R.lo[0] && ix < R.hi[0] && iy >= R.lo[1] && iy < R.hi[1] && iz >= R.lo[2] && iz < R.hi[2]) continue;
+        const float rho = __ldg(grid + ix + (int64_t)nx * (iy + (int64_t)ny * iz));
+        Pair d[3], sq[3];
+        for (int k = 0; k < 3; ++k) {
+            d[k] = add(R.d0[k], mul({(float)c[k], 0.0f}, R.step[k]));
+            sq[k] = rounded(mul(d[k], d[k]));
+        }
+        float f, g;
+        series_lacks(sp, sp4, sq[0], sq[1], sq[2], f, g);
+        sum.x = fmaf(rho, f, sum.x);
+        sum.y = fmaf(rho * d[2].h, g, sum.y);
+    }
+    return sum;
+}
 
 template <bool CUBE>
 __global__ void __launch_bounds__(kFieldThreads, 2) field_voxel_kernel(const FieldParams P)
@@ -145,7 +179,9 @@ __global__ void __launch_bounds__(kFieldThreads, 2) field_voxel_kernel(const Fie
     const int parts = (int)cluster.num_blocks(), part = (int)cluster.block_rank();
     __shared__ float tile[kFieldThreads][kFieldCols + 1];
     __shared__ Pair sx[kFieldCols];     // X of the tile's columns
-    __shared__ float sp[kFieldTerms];   // the series for lengths in units of L
+    __shared__ Pair sp4[6];  
+    __shared__ Rim rim;
+    __shared__ float sp[kSeriesTerms];   // the series for lengths in units of L
     __shared__ double red[2][kFieldThreads / 32], total[2];
     const int64_t i = blockIdx.x / parts;
     const int t = threadIdx.x;
@@ -168,9 +204,11 @@ __global__ void __launch_bounds__(kFieldThreads, 2) field_voxel_kernel(const Fie
     if (none_near)
         for (int k = 0; k < 3; ++k) lo[k] = hi[k] = 0;
     const double L = sqrt(fmax(sqrt(out2), P.near) * sqrt(far2)), invL = 1.0 / L;
-    if (t < kFieldTerms) {
-        const double q = invL * invL;
-        sp[t] = (float)(P.series[t] * (t < 3 ? q : t < 9 ? q * q : t < 19 ? q * q * q : (q * q) * (q * q)));
+    if (t < kSeriesTerms) {
+        const double q = invL * invL, q2 = q * q;
+        const double v = P.series[t] * (t < 3 ? q : t < 9 ? q2 : t < 19 ? q2 * q : t < 34 ? q2 * q2 : q2 * q2 * q);
+        sp[t] = (float)v;
+        if (t >= 3 && t < 9) sp4[t - 3] = pair_of(v);
     }
 
     // far cells: sum of rho f and of rho (df/dz), lengths in units of L
@@ -233,6 +271,23 @@ __global__ void __launch_bounds__(kFieldThreads, 2) field_voxel_kernel(const Fie
         }
         phi += (double)fs.h + (double)fs.l;
         gz += dz * ((double)gs.h + (double)gs.l);
+    }
+    if (t >= 64 && t < 67) {  // (a thread per axis: all of them would wait for the double-precision pipe)
+        const int k = t - 64, nk = k == 0 ? P.nx : (k == 1 ? P.ny : P.nz);
+        const double xk = P.x[3 * i + k], a = (xk - P.org[k]) / P.sp[k], w = P.near * (kRimCells / kNearCells) / P.sp[k];
+        const int first = (int)fmin(fmax(ceil(a - w - 0.5), 0.0), (double)nk);
+        rim.first[k] = first;
+        rim.count[k] = max((int)fmin(fmax(floor(a + w - 0.5) + 1.0, 0.0), (double)nk) - first, 0);
+        rim.lo[k] = k == 0 ? lo[0] : (k == 1 ? lo[1] : lo[2]);
+        rim.hi[k] = k == 0 ? hi[0] : (k == 1 ? hi[1] : hi[2]);
+        rim.d0[k] = pair_of((P.org[k] + (first + 0.5) * P.sp[k] - xk) * invL);
+        rim.step[k] = pair_of(P.sp[k] * invL);
+    }
+    __syncthreads();  // (sp: a block may have had no rows)
+    {
+        const float2 lacks = rim_sum(P.grid, P.nx, P.ny, rim, sp, sp4, part * kFieldThreads + t, parts * kFieldThreads);
+        phi += (double)lacks.x;
+        gz += (double)lacks.y;
     }
     const double V = P.sp[0] * P.sp[1] * P.sp[2];
     phi *= V * invL;
@@ -460,9 +515,7 @@ extern "C" int mcg_field(const mcg_density* density, const double* points_dev, i
             P.sp[k] = density->spacing[k];
         }
         const double half[3] = {0.5 * P.sp[0], 0.5 * P.sp[1], 0.5 * P.sp[2]};
-        double series[kSeriesTerms];
-        cell_series(half, series);
-        std::memcpy(P.series, series, sizeof(P.series));
+        cell_series(half, P.series);
         P.near = kNearCells * std::max(P.sp[0], std::max(P.sp[1], P.sp[2]));
         // few points: a cluster of eight blocks each, so that they fill the SMs
         const unsigned parts = n < 2048 ? 8u : 1u;

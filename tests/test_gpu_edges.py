@@ -4,6 +4,7 @@
 * double-precision normals: every digit of the small ones too;
 * a density that is not finite: only the walks that meet it;
 * boundary tables: grids of many cells in a row; near zones of a few cells;
+* the field of small grids to the last digits that doubles hold;
 * an error of one launch is not reported by the next;
 * mcgrav_solve: its workspace goes back, and a failed call waits as well;
 * mcgrav_solve after a device reset;
@@ -262,3 +263,48 @@ def test_solve_after_a_device_reset():
     r = subprocess.run([sys.executable, "-c", RESET], cwd=root, env=dict(os.environ, CUDART=cudart(), PYTHONPATH=root),
                        capture_output=True, text=True, timeout=120)
     assert r.returncode == 0, r.stderr
+
+
+def field_in_long_doubles(w, grid, points):
+    """dPhi/dz by node sums in numpy's long doubles (64-bit mantissa or more), and
+    the sum of the cells' own magnitudes."""
+    L = np.longdouble
+    nz, ny, nx = grid.shape
+    weight = np.zeros((nz + 1, ny + 1, nx + 1), L)
+    for m in range(8):
+        i, j, k = m & 1, m >> 1 & 1, m >> 2
+        weight[k:k + nz, j:j + ny, i:i + nx] += grid.astype(L) * (1 if (i + j + k) & 1 else -1)
+    x, y, z = (L(w.grid_origin[a]) + np.arange(n + 1, dtype=L) * L(w.grid_spacing[a]) for a, n in
+               enumerate((nx, ny, nz)))
+    gz, size = [], []
+    for p in points:
+        a, b, c = (x - L(p[0]))[None, None, :], (y - L(p[1]))[None, :, None], (z - L(p[2]))[:, None, None]
+        r = np.sqrt(a * a + b * b + c * c)
+
+        def ln(t, s2):      # ln(t + r), without cancellation
+            t = t + 0 * r
+            return np.where(t < 0, np.log(s2 + 0 * r) - np.log(r + np.abs(t)), np.log(r + np.abs(t)))
+
+        D = a * ln(b, a * a + c * c) + b * ln(a, b * b + c * c) - c * np.arctan(a * b / (c * r))
+        gz.append(float(w.G * np.sum(weight * D)))
+        mid = [(v[1:] + v[:-1]) / 2 for v in (a.ravel(), b.ravel(), c.ravel())]
+        r2 = mid[0][None, None, :] ** 2 + mid[1][None, :, None] ** 2 + mid[2][:, None, None] ** 2
+        size.append(float(w.G * np.prod(w.grid_spacing) * np.sum(np.abs(grid) / r2)))
+    return np.array(gz), np.array(size)
+
+
+@pytest.mark.parametrize("shape", [(20, 17, 9), (16, 16, 8), (31, 19, 8)])
+def test_field_of_small_grids_over_their_surface(shape):
+    """Where single-precision terms of few cells weigh most.  Bound: 3e-14 for the
+    pairs (2^-45 of every cell), 1.2e-13 for the cancellation of the near nodes in
+    doubles (their terms are some 500 times the cells'), 5e-14 for what remains of
+    the series (1e-12 of the cells beyond the rim, a twentieth of the sum)."""
+    w = W.voxel_survey(shape=shape).with_(g_kind="zero")
+    rng = np.random.default_rng(5)
+    grid = (300.0 * np.expm1(rng.normal(size=shape[::-1]))).astype(np.float32)
+    pts = rng.uniform(w.lo, w.hi, (40, 3))
+    pts[:, 2] = 0.01 * np.abs(pts[:, 2])
+    out = torch.empty((2, 40), dtype=torch.float64, device="cuda")
+    M.mcg_field(M.problem(w, grid=torch.from_numpy(grid).cuda()), torch.from_numpy(pts).cuda(), 40, out[0], out[1])
+    want, size = field_in_long_doubles(w, grid, pts)
+    assert np.all(np.abs(out[1].cpu().numpy() - want) <= 2e-13 * size)
