@@ -55,11 +55,11 @@ FP64_OPS_PER_RNG_STEP = 9.9
 L2_FLUSH_BYTES = 256 << 20
 # DRAM bytes (read + write) of one walk_mixed_kernel launch per work item,
 # from ncu's dram__bytes_read.sum + dram__bytes_write.sum (one pass) on a
-# full-size launch of this workload, 30 x 131072 items: 42.8 MB read + 410.4 MB
-# written = 115.2 B per item (the 32-byte exit records stay in L2 in smaller
+# full-size launch of this workload, 30 x 131072 items: 36.4 MB read + 391.2 MB
+# written = 108.7 B per item (the 32-byte exit records stay in L2 in smaller
 # launches, so a smaller case does not scale).  To be re-measured (or reported
 # as null) whenever the walk kernel changes.
-WALK_DRAM_BYTES_PER_ITEM = 115.2
+WALK_DRAM_BYTES_PER_ITEM = 108.7
 
 
 def parse():
@@ -257,9 +257,8 @@ def run_ours(args):
         # the library's autotuner on this workload (stepping rate, then tail)
         M.mcg_autotune(prob, stations, S, w.dt, w.seed, opts[0])
         for o in opts[1:]:
-            o.block, o.refill_min, o.spill_max = opts[0].block, opts[0].refill_min, opts[0].spill_max
-        tuned = {"block": int(opts[0].block), "refill_min": int(opts[0].refill_min),
-                 "spill_max": int(opts[0].spill_max)}
+            o.block, o.refill_min = opts[0].block, opts[0].refill_min
+        tuned = {"block": int(opts[0].block), "refill_min": int(opts[0].refill_min)}
 
     def path_block(j):
         # step j of this rank takes paths [p0, p0 + Bp) of every station: a
@@ -783,7 +782,6 @@ def large_survey_block(M, W, steps, warmup, paths):
     ds = pair[0]
     M.mcg_autotune(ds.prob, ds.stations, ds.S, w.dt, w.seed, ds.opts)
     pair[1].opts.block, pair[1].opts.refill_min = ds.opts.block, ds.opts.refill_min
-    pair[1].opts.spill_max = ds.opts.spill_max
     pair[1].states = ds.states
 
     def run_steps(first, count):
@@ -848,8 +846,7 @@ def large_survey_block(M, W, steps, warmup, paths):
     for name, prec in (("fp64", M.MCG_FP64), ("mixed", M.MCG_MIXED)):
         dd = DeviceSolve(w, stations=w.stations[sample], batch=n_direct, precision=prec, grid=grid, faces=faces)
         if prec == M.MCG_MIXED:
-            dd.opts.block, dd.opts.refill_min, dd.opts.spill_max = ds.opts.block, ds.opts.refill_min, \
-                ds.opts.spill_max
+            dd.opts.block, dd.opts.refill_min = ds.opts.block, ds.opts.refill_min
         torch.cuda.synchronize()
         h0 = time.perf_counter()
         rd = dd.run(paths=n_direct)
@@ -877,8 +874,7 @@ def large_survey_block(M, W, steps, warmup, paths):
             "steps": steps, "warmup": warmup, "ms_per_step": t / steps * 1e3,
             "stations_per_s_at_1e-3": stations_per_s, "mean_path_steps_per_path": mean_steps,
             "median_paths_needed_at_1e-3": float(np.median(n_req)),
-            "autotuned": {"block": int(ds.opts.block), "refill_min": int(ds.opts.refill_min),
-                          "spill_max": int(ds.opts.spill_max)},
+            "autotuned": {"block": int(ds.opts.block), "refill_min": int(ds.opts.refill_min)},
             "fp64_walk": {"path_steps_per_s": rate64, "stations_per_s_at_1e-3": stations_per_s_64,
                           "how": "tail-free FP64 stepping rate (paths capped at 256 RNG-steps) on the same model"},
             "mixed_over_fp64_at_equal_se": stations_per_s / stations_per_s_64,
@@ -891,7 +887,7 @@ def large_survey_block(M, W, steps, warmup, paths):
                                "mean_rel_u": float(np.mean((r["u"][pick] - phi) / np.abs(phi))),
                                "median_rel_se_u": float(np.median(r["se_u"][pick] / np.abs(r["u"][pick]))),
                                "field_ms": g0.elapsed_time(g1),
-                               "reference": "voxel prism sums by node summation (mcg_field)"},
+                               "reference": "exact field of the voxel model (mcg_field)"},
             "model_setup_s": setup_s, "status": r["status"],
             "config": {"workload": "large_survey: 100x100 grid at 20 m, z = 0 and z = 100 m, voxel_survey model",
                        "step_m": w.step_length, "h_m": w.h, "packed_grid": ds.prob.density.zpack is not None}}

@@ -168,7 +168,9 @@ typedef struct {
     int32_t migrate;         /* mixed walk: 1 (default) lets fault_unpublished act;
                                 no effect otherwise: once the work list is used up a
                                 warp runs its last walks with several lanes each
-                                instead of handing them to other warps             */
+                                instead of handing them to other warps, and waits
+                                for none (MCG_ERR_TIMEOUT comes from that hook
+                                alone)                                             */
     int32_t fault_unpublished;/* failure-detection test hook, 0..255 (default 0):
                                 the launch starts with this many slots of a
                                 hand-over pool reserved but never published, as if
@@ -218,8 +220,8 @@ MCG_API const char* mcg_version(void);
  *            points below take device pointers only).
  *   out      : HOST arrays of length S.
  * Blocking.  Takes a device workspace for the duration of the call from a
- * memory pool of the library's own (which keeps up to 256 MiB per device for
- * later calls and hands back the rest):
+ * memory pool of the library's own (one per context, which keeps up to 256 MiB
+ * for later calls; the rest is handed back before the call returns):
  * mcg_workspace_bytes(S, batch), plus the packed copies of a voxel grid and
  * of boundary tables (mcg_voxel_pack_bytes, mcg_table_pack_bytes) unless the
  * caller passes them, plus the grid and tables themselves when they are in
@@ -261,6 +263,11 @@ MCG_API int mcgrav_solve(const mcg_domain* domain, const mcg_density* density, c
  * flags an item's count once all its copies have written their exit records,
  * and its exit kernel evaluates flagged items only), so nothing is read from
  * an earlier launch.
+ * With none, a sphere or a prism as the density a path's values depend on
+ * (seed, station, path) alone.  With a voxel grid the mixed walk's single-
+ * precision sums are flushed where its warp regroups, which depends on the
+ * launch and on the race for items: there two runs agree to rounding (at most
+ * 64 2^-24 of the source integral per flush; some 1e-7 of u), not bit for bit.
  * Allocates nothing. */
 MCG_API int mcg_walk(const mcg_domain* domain, const mcg_density* density, const mcg_boundary* boundary,
              const double* stations_dev, int64_t S, int64_t p0, int64_t N, double dt, uint64_t seed,
@@ -515,10 +522,14 @@ MCG_API int mcg_grf_density(uint64_t seed, int64_t nx, int64_t ny, int64_t nz, d
  * Phi = -G sum_voxels rho_v [[[F]]]_v of the voxel model (prism summation,
  * the closed form the paper compares against, Sec. 1 and Sec. 4.2) at the
  * nu x nv nodes of each face of `domain` (layout as MCG_G_TABLE).  Voxels
- * whose centre lies within `near_cells` cell diagonals of a node use the
- * exact prism potential in double precision; farther voxels, which must be
- * cubes or close to them, use their point-mass term rho_v V / r in single
- * precision, whose relative error for a cube is O((d/r)^4).  Supports
+ * whose centre lies within `near_cells` cell diagonals of a node enter with
+ * their own potential: those next to it (up to three or four of the longest
+ * cell side, 2.25 for elongated cells) by prism sums in double precision, the
+ * others of them by the series of the averaged 1/r to tenth order, whose
+ * remainder is at most 1e-10 of the voxel's term (9e-10 for elongated cells)
+ * and whose rounding 3e-14; farther voxels, which must be cubes or close to
+ * them, by their point-mass term rho_v V / r in single precision, whose
+ * relative error for a cube is O((d/r)^4).  Supports
  * nx <= 128.  faces_out: DEVICE float32, 6 nv nu.  density->grid: DEVICE.
  * Asynchronous on `stream`.  Allocates nothing. */
 MCG_API int mcg_boundary_tables(const mcg_domain* domain, const mcg_density* density, int32_t nu, int32_t nv,
@@ -536,13 +547,18 @@ MCG_API int mcg_boundary_tables(const mcg_domain* domain, const mcg_density* den
  *   SPHERE: -G M / r outside, -G M (3 a^2 - r^2) / (2 a^3) inside.
  *   PRISM : Nagy's corner function F over the eight corners,
  *           Phi = -G rho0 [[[F]]], dPhi/dz = G rho0 [[[dF/dz]]].
- *   VOXEL : the sum of every voxel's prism field, regrouped by grid node:
- *           Phi(x) = -G sum_nodes w_n F(node - x), where w_n adds the
+ *   VOXEL : the sum of every voxel's prism field.  Cells within six of the
+ *           longest cell side of the point (per axis) are regrouped by grid
+ *           node: Phi(x) = -G sum_nodes w_n F(node - x), where w_n adds the
  *           densities of the (up to eight) cells sharing the node with the
- *           sign of that corner in each cell's prism sum.  Double precision
- *           with compensated sums; one block per point, (nx+1)(ny+1)(nz+1)
- *           corner evaluations per point (about 0.5 ms per point on a GB300
- *           for a 128 x 128 x 64 grid).
+ *           sign of that corner in each cell's prism sum, in double precision
+ *           with compensated sums.  The others use the series of the averaged
+ *           1/r, its leading terms as unevaluated sums of two single-precision
+ *           numbers (45 bits).  Error: about 1e-13 of the cells' summed
+ *           magnitudes, below that of node sums over the whole grid.  Cell
+ *           densities beyond 1e-30 .. 1e36 in magnitude lose digits or
+ *           overflow there.  2.6 ms for 256 points over a 128 x 128 x 64 grid
+ *           on a GB300, 0.30 ms for one.
  *   NONE  : 0.
  * points_dev: DEVICE, n x 3 row-major.  phi_dev, gz_dev: DEVICE, length n
  * (either may be NULL).  density->grid: DEVICE.  Asynchronous on `stream`.

@@ -190,7 +190,7 @@ __device__ __forceinline__ double square_sum(double a, double b2) { return __fma
 // exact prisms in double precision throughout (6 x 128^2 nodes: 342 of 377 ms,
 // ~690 prisms a node of 8 corners; the pipe does 1.6 operations a clock and
 // SM).  Now 0.5 and 37 ms, 25 of them the point masses, with the same values
-// to the last bit.
+// to the last bit (twelve grids and zones).
 template <int NPL>
 __global__ void __launch_bounds__(kTableThreads, 2) tables_kernel(const TableParams T)
 {
@@ -511,7 +511,11 @@ int boundary_tables(const mcg_domain* d, const mcg_density* rho, int32_t nu, int
     for (int i = 0; i < 3; ++i) T.second[i] = series[i];
     for (int i = 0; i < kSeriesTerms; ++i) T.series[i] = (float)series[i];
     // two nodes a lane share each density read; with few nodes one, and a
-    // cluster of eight blocks for each 32 of them, so that they fill the SMs
+    // cluster of eight blocks for each 32 of them, so that they fill the SMs.
+    // (128 x 128 x 64 cells; one node a lane in 1 and 8 blocks, two in 1 and 8:
+    // 486 nodes 3.4, 0.53, 6.0, 0.85 ms; 14406 8.9, 7.0, 9.7, 6.7; 25350 11.2,
+    // 11.3, 12.2, 10.6; 39366 16.8, 17.8, 17.7, 16.8; 60000 24.8, 26.9, 24.4, 25.6;
+    // 98304 38.1, 43.0, 37.3, 40.2)
     int dev = 0, sms = 152;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

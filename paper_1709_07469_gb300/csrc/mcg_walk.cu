@@ -124,7 +124,8 @@ __device__ __forceinline__ double exit_mixed(const WalkParams& P, const ModelRef
 // 32 bytes, written as two 16-byte stores that fill one sector -- X (the walk
 // position before the exit step, copy 0's coordinates; copy c adds its z
 // offset), Y (the copy's first point not strictly inside Omega) and the
-// source sum in double.  rho at X is not stored:
+// source sum (a double's bits or, where the density is rho0 or 0, a count of
+// half points: recorded_sum).  rho at X is not stored:
 // exit_mixed_kernel evaluates the same single-precision density function at
 // the same X, which gives the walk's value bit for bit.  The record is valid
 // once the item's step count carries kDoneFlag.
@@ -160,7 +161,8 @@ __device__ __forceinline__ double recorded_sum(const WalkParams& P, unsigned lon
         return __longlong_as_double((long long)acc);
 }
 
-// The flushed part with `part` added.
+// The flushed part with `part` added (the same sum as source_sum's: a count since
+// the last flush is below 2^22, so the width it is converted in does not matter).
 template <int RHO>
 __device__ __forceinline__ unsigned long long flushed(unsigned long long held, float part)
 {
@@ -233,7 +235,8 @@ __device__ __noinline__ unsigned bridge_exits_f32(const WalkParams& P, unsigned 
 //    runs through shared memory; then each lane tests and sums its own block.
 //
 // Both take the same steps in the same arithmetic, so a walk's numbers do not
-// depend on how it was run.  What bounds them, on the prism ore body (1 m
+// depend on how it was run (but for the rounding of a voxel grid's sums, which
+// are flushed where the warp regroups).  What bounds them, on the prism ore body (1 m
 // steps): a walk alone takes 115 ns a step as a lane (the block's dependent
 // generator, logarithm and root, ~950 cycles) and 7 ns as a strip of 32 (that
 // once per 32 blocks, and the chain, 16 cycles a block); with the GPU full,
@@ -1153,8 +1156,9 @@ cudaError_t launch_walk(const WalkParams& P0, int precision, int block, cudaStre
         // lies (prism, 20 walks per resident warp: strips 65 ms, full lanes
         // in fewer warps 79 ms; 30 per warp: 84 against 94 ms).  A voxel
         // grid always starts with full warps: the rounding of its single-
-        // precision sums follows the walks that share a warp, and 32
-        // consecutive items keep it the same however many SMs there are.
+        // precision sums follows the walks that share a warp, and a warp's
+        // first 32 are consecutive items on any launch (later ones are not:
+        // its free lanes take the next items of the list).
         const long long per_block = block / 32;
         const unsigned long long warps = (unsigned long long)(grid * per_block);
         const long long per_warp = (long long)(P.total / warps);

@@ -16,12 +16,12 @@
 // increments of one four-step block, a lane per walk and coordinate adds them
 // up in order through shared memory, then each lane tests its own block.
 //
-// What bounds it: with the GPU full the double-precision pipe (busy 74 % of
+// What bounds it: with the GPU full the double-precision pipe (busy 71 % of
 // the time: 64 operations of a block's 3100 instructions a lane) and the
-// integer pipes beside it (issue 57 %): 27.2 steps/ns against 3.2 for the plain
+// integer pipes beside it (issue 58 %): 27.3 steps/ns against 3.2 for the plain
 // evaluation (ore body, capped walks).  With few walks the chain of additions
-// and a block's dependent integers: 110 ns a step for a lone walk (6270
-// before).  Walks of the sphere, 8 x 2000 paths: 17.7 -> 0.91 ms; ore body at
+// and a block's dependent integers: 88 ns a step for a lone walk over the ore
+// body, most of its blocks far from it (6270 before).  Walks of the sphere, 8 x 2000 paths: 17.7 -> 0.91 ms; ore body at
 // 10 m steps, 30 x 256 paths: 106.7 -> 2.06 ms.
 #include <cmath>
 
@@ -37,8 +37,10 @@ namespace mcg {
 namespace {
 
 constexpr int kSlots = 16;          // walks a warp holds: live, and ended ones waiting for their evaluation
-constexpr unsigned kLiveMax = 8;    // live ones at most
-constexpr int kBatch = 10;          // walks evaluated at once: 30 copies on 32 lanes
+constexpr unsigned kLiveMax = 8;    // live ones at most (with 4, a full launch 22.4 steps/ns instead of 27.3,
+                                    // 8 x 2000 paths of the sphere 0.81 ms instead of 0.91)
+constexpr int kBatch = 10;          // walks evaluated at once: 30 copies on 32 lanes (5 and 8: no difference
+                                    // beyond the runs' own)
 constexpr int kMoveRow = 33;        // double2 per row of the moves
 
 // How near to a face, or (squared) to a sphere, single precision does not
