@@ -113,13 +113,15 @@ __device__ __forceinline__ float series_value(float P4, float P6, float P8, floa
     return y4 * y4 * y * fmaf(y4, fmaf(y4, P8, P6), P4);
 }
 
-// P_10 y^21.
+// P_10, and P_10 y^21.
+__device__ __forceinline__ float series_p10(const float* p, const SeriesRow& r, float X)
+{
+    return fmaf(fmaf(fmaf(fmaf(fmaf(p[34], X, r.c10[0]), X, r.c10[1]), X, r.c10[2]), X, r.c10[3]), X, r.c10[4]);
+}
 __device__ __forceinline__ float series_tenth(const float* p, const SeriesRow& r, float X, float y, float y2)
 {
-    const float P10 = fmaf(fmaf(fmaf(fmaf(fmaf(p[34], X, r.c10[0]), X, r.c10[1]), X, r.c10[2]), X, r.c10[3]), X,
-                           r.c10[4]);
     const float y4 = y2 * y2, y8 = y4 * y4;
-    return y8 * y8 * y4 * y * P10;
+    return y8 * y8 * y4 * y * series_p10(p, r, X);
 }
 
 // The same terms (n = 2, 3, 4) of (df/dz) / d_z: 2 dP_2n/dZ y^(4n+1) - (4n+1) P_2n y^(4n+3);
@@ -180,15 +182,19 @@ __device__ __forceinline__ void series_lacks(const float* p, const Pair* p4, Pai
     const float v = series_value(P4, P6, P8, y.h, y2.h), s = series_slope(p, r, X.h, P4, P6, P8, y.h, y2.h);
     const float y4 = y2.h * y2.h, y13 = y4 * y4 * y4 * y.h;
     const float v68 = y13 * fmaf(y4, P8, P6), s68 = y13 * slope_rest(p, r, X.h, P6, P8, y2.h);
-    // P_10
-    const float *q = p + 34, Zd = Z.h * Z.h, Zt = Zd * Z.h;
-    const float d3 = fmaf(q[4], Y.h, 2.0f * q[5] * Z.h);
-    const float d2 = fmaf(fmaf(q[7], Y.h, 2.0f * q[8] * Z.h), Y.h, 3.0f * q[9] * Zd);
-    const float d1 = fmaf(fmaf(fmaf(q[11], Y.h, 2.0f * q[12] * Z.h), Y.h, 3.0f * q[13] * Zd), Y.h, 4.0f * q[14] * Zt);
-    const float d0 = fmaf(fmaf(fmaf(fmaf(q[16], Y.h, 2.0f * q[17] * Z.h), Y.h, 3.0f * q[18] * Zd), Y.h,
-                               4.0f * q[19] * Zt), Y.h, 5.0f * q[20] * Zd * Zd);
-    const float D10 = fmaf(fmaf(fmaf(fmaf(q[2], X.h, d3), X.h, d2), X.h, d1), X.h, d0);
-    const float v10 = series_tenth(p, r, X.h, y.h, y2.h), s10 = fmaf(2.0f * D10, y13 * y4 * y4, -21.0f * y2.h * v10);
+    // P_10 and 2 dP_10/dZ - 21 P_10 y^2, of the direction: homogeneous of degree 5 and
+    // 4, so that no power above y^13 is formed (in a long grid y is 100 and more)
+    const float x1 = X.h * y2.h, y1 = Y.h * y2.h, z1 = Z.h * y2.h, z2 = z1 * z1, z3 = z2 * z1;
+    const SeriesRow u = series_row(p, y1, z1);
+    const float* q = p + 34;
+    const float d3 = fmaf(q[4], y1, 2.0f * q[5] * z1);
+    const float d2 = fmaf(fmaf(q[7], y1, 2.0f * q[8] * z1), y1, 3.0f * q[9] * z2);
+    const float d1 = fmaf(fmaf(fmaf(q[11], y1, 2.0f * q[12] * z1), y1, 3.0f * q[13] * z2), y1, 4.0f * q[14] * z3);
+    const float d0 = fmaf(fmaf(fmaf(fmaf(q[16], y1, 2.0f * q[17] * z1), y1, 3.0f * q[18] * z2), y1,
+                               4.0f * q[19] * z3), y1, 5.0f * q[20] * z2 * z2);
+    const float D10 = fmaf(fmaf(fmaf(fmaf(q[2], x1, d3), x1, d2), x1, d1), x1, d0);
+    const float P10 = series_p10(p, u, x1);
+    const float v10 = y4 * y4 * y2.h * y.h * P10, s10 = y13 * fmaf(-21.0f, P10, 2.0f * D10);
     // P_4 and 2 dP_4/dZ - 9 P_4 y^2
     const Pair a = add(mul(p4[1], Y), mul(p4[2], Z));
     const Pair b = add(mul(add(mul(p4[3], Y), mul(p4[4], Z)), Y), mul(mul(p4[5], Z), Z));

@@ -4,7 +4,7 @@
 * double-precision normals: every digit of the small ones too;
 * a density that is not finite: only the walks that meet it;
 * boundary tables: grids of many cells in a row; near zones of a few cells;
-* the field of small grids to the last digits that doubles hold;
+* the field of small grids to the last digits that doubles hold; of long ones;
 * an error of one launch is not reported by the next;
 * mcgrav_solve: its workspace goes back, and a failed call waits as well;
 * mcgrav_solve after a device reset;
@@ -308,3 +308,31 @@ def test_field_of_small_grids_over_their_surface(shape):
     M.mcg_field(M.problem(w, grid=torch.from_numpy(grid).cuda()), torch.from_numpy(pts).cuda(), 40, out[0], out[1])
     want, size = field_in_long_doubles(w, grid, pts)
     assert np.all(np.abs(out[1].cpu().numpy() - want) <= 2e-13 * size)
+
+
+@pytest.mark.parametrize("shape", [(1, 20000, 1), (1, 65534, 1), (40000, 1, 2)])
+def test_field_of_long_grids(shape):
+    """Rows of up to 65534 cubes, points over and beside them.  Reference: prism
+    sums for the cells within 64 sides, point masses for the others (the next term
+    of a cube: 0.2 (1 / 128)^4 of its own, 1e-9)."""
+    w = box_of_cells(shape, 10.0)
+    axis = int(np.argmax(shape))
+    grid = np.random.default_rng(axis).uniform(100.0, 500.0, shape[::-1]).astype(np.float32)
+    pts = np.zeros((12, 3))
+    pts[:, axis] = 10.0 * np.array([0.0, 3.3, 7000.4, -0.5 * shape[axis] + 2.0] * 3)
+    pts[:, 2] += np.repeat([12.0, 71.0, 300.0], 4)
+    out = torch.empty((2, 12), dtype=torch.float64, device="cuda")
+    M.mcg_field(M.problem(w, grid=torch.from_numpy(grid).cuda()), torch.from_numpy(pts).cuda(), 12, out[0], out[1])
+    got = out.cpu().numpy()
+    c = [(w.lo[k] + 10.0 * (np.arange(shape[k]) + 0.5)).reshape([-1 if 2 - k == d else 1 for d in range(3)])
+         for k in range(3)]
+    to = [1] * 3
+    to[2 - axis] = -1
+    for i, x in enumerate(pts):
+        near = np.abs(c[axis].ravel() - x[axis]) < 640.0
+        part = np.where(near.reshape(to), grid, 0).astype(np.float32)
+        phi, gz = oracle.voxel_field(oracle_spec(w, grid=part), x[None, :], threads=THREADS, want_gz=True)
+        far = np.where(near.reshape(to), 0.0, grid.astype(np.float64))
+        r = np.sqrt((c[0] - x[0]) ** 2 + (c[1] - x[1]) ** 2 + (c[2] - x[2]) ** 2)
+        np.testing.assert_allclose(got[0, i], phi[0] - w.G * 1000.0 * np.sum(far / r), rtol=1e-8)
+        np.testing.assert_allclose(got[1, i], gz[0] - w.G * 1000.0 * np.sum(far * (c[2] - x[2]) / r**3), rtol=1e-8)
